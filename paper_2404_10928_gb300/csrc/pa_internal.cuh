@@ -294,6 +294,9 @@ cudaError_t launch_build_table(int dim, TileRef* table, int2* krange, const doub
 cudaError_t launch_fwd_copies(int dim, unsigned long long* copies, TileRef* table,
                               const double* sensors_dev, int S, const pa_grid& grid, const GridF& g,
                               double kappa, int L, cudaStream_t st);
+// the combine's tables from the reference table: sorted and upper of FwdParams
+cudaError_t launch_combine_order(const TileRef* table, int2* sorted, int* upper, int S, int K, int L,
+                                 int ntiles, cudaStream_t st);
 cudaError_t launch_pack(const float* r, float2* packed, int S, int K, int Kp, int pad,
                         cudaStream_t st);
 cudaError_t launch_bp_filter(const float* p, float2* packed, int S, int K, int Kp, int pad,

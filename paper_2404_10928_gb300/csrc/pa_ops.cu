@@ -535,6 +535,91 @@ cudaError_t launch_build_table(int dim, TileRef* table, int2* krange, const doub
                   err);
 }
 
+// Combine order of one sensor per CTA: its tiles that are not skipped sorted by
+// window start (ties by tile index), and for every sample k the number of windows
+// starting at or before k.  A counting sort in the row of `upper` itself: entry
+// klo + L counts the windows starting at klo, an exclusive scan turns the counts
+// into first positions, and the scatter (one warp, tiles in index order, equal
+// starts ranked by a match) advances each to its end, which is the inclusive
+// count wanted.  The row is staged in shared memory when it fits (`staged`).
+// Bounded by latency (a few dependent passes over a few thousand entries per
+// sensor).  The host sort with its three copies that this replaces took most of
+// pa_plan_set_sound_speed: 0.40 -> 0.08 ms at 256^2 with 128 sensors, 95 -> 9.6 ms at
+// 128^3 with 1024 (creating that plan: 97 -> 11 ms).
+constexpr int kOrderThreads = 256;
+constexpr int kOrderStaged = 12 * 1024;  // entries (48 KB)
+__global__ void __launch_bounds__(kOrderThreads) k_combine_order(const TileRef* table, int2* sorted,
+                                                                 int* upper, int S, int K, int L,
+                                                                 int ntiles, int staged) {
+  extern __shared__ int s_row[];
+  __shared__ int s_warp[kOrderThreads / 32];
+  const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = K + L;
+  int* out = upper + (int64_t)s * n;
+  int* row = staged ? s_row : out;
+  for (int j = tid; j < n; j += kOrderThreads) row[j] = 0;
+  __syncthreads();
+  // starts lie in (-L, K): a window that is not skipped meets [0, K)
+  auto start = [&](int t) {
+    const int klo = table[(int64_t)t * S + s].klo;
+    const int j = klo == kSkip ? -1 : window_start(klo) + L;
+    return j < n ? j : -1;
+  };
+  for (int t = tid; t < ntiles; t += kOrderThreads) {
+    const int j = start(t);
+    if (j >= 0) atomicAdd(&row[j], 1);
+  }
+  __syncthreads();
+  // exclusive scan: a contiguous share per thread
+  const int per = (n + kOrderThreads - 1) / kOrderThreads;
+  const int j0 = min(n, tid * per), j1 = min(n, j0 + per);
+  int sum = 0;
+  for (int j = j0; j < j1; ++j) sum += row[j];
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  int base = incl - sum;
+  for (int w = 0; w < warp; ++w) base += s_warp[w];
+  for (int j = j0; j < j1; ++j) {
+    const int v = row[j];
+    row[j] = base;
+    base += v;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int2* dst = sorted + (int64_t)s * ntiles;
+    for (int t0 = 0; t0 < ntiles; t0 += 32) {
+      const int t = t0 + lane;
+      const int j = t < ntiles ? start(t) : -1;
+      const unsigned same = __match_any_sync(0xffffffffu, j);
+      if (j >= 0) {
+        const int pos = row[j] + __popc(same & ((1u << lane) - 1u));
+        dst[pos] = make_int2(t, j - L);
+      }
+      __syncwarp();
+      if (j >= 0 && lane == __ffs(same) - 1) row[j] += __popc(same);
+      __syncwarp();
+    }
+  }
+  if (staged) {
+    __syncthreads();
+    for (int j = tid; j < n; j += kOrderThreads) out[j] = row[j];
+  }
+}
+
+cudaError_t launch_combine_order(const TileRef* table, int2* sorted, int* upper, int S, int K, int L,
+                                 int ntiles, cudaStream_t st) {
+  const int staged = K + L <= kOrderStaged;
+  return launch_k(k_combine_order, dim3(S), dim3(kOrderThreads),
+                  staged ? (size_t)(K + L) * sizeof(int) : 0, st, 0, table, sorted, upper, S, K, L,
+                  ntiles, staged);
+}
+
 // ---------------------------------------------------------------------------
 // trace packing: r[s][k] -> packed[s][pad + k] = (mid, slope) for k in [-1, K),
 // mid = (r_k + r_{k+1})/2, slope = r_{k+1} - r_k, with r_{-1} = r_K = 0.
@@ -984,9 +1069,12 @@ int forward_smem_bytes(int dim, int L, int spc) {
 // l), so every warp atomic of the gather is one row.
 //   Copies: lanes l = 0..31 in turn take the copy c whose bank (bin + c
 // kFwdCopyRes) mod 32 minimises, summed over the 32 rows, the squared number
-// of lanes already assigned to that bank (ties to the lower copy).  Bins come
-// from FP32 distances: an occasional bin off by one costs at most a bank
-// conflict.  Output: copies[tile * S + s], 2 bits per lane.
+// of lanes already assigned to that bank (ties to the lower copy; two
+// candidates' sums, each at most 32 x 31^2 < 2^16, share a warp reduction: the
+// reductions bound the kernel, which took 104 us with one per candidate for the
+// 256^2 ring with 256 sensors and takes 72 us).  Bins come from FP32 distances:
+// an occasional bin off by one costs at most a bank conflict.  Output:
+// copies[tile * S + s], 2 bits per lane.
 //   Tap scale: a window sample receives one tap from every pixel whose arrival
 // u lies within one sample of it.  The warp counts, per sample, the pixels with
 // u within 1 + kTapSlack samples (the slack covers the FP32 distances here
@@ -1046,11 +1134,12 @@ __global__ void __launch_bounds__(256) k_fwd_copies(unsigned long long* copies, 
     for (int l = 0; l < 32; ++l) {
       const int lo = (int)floorf(uf[l] - kTapSlack) - bmin;
       const int hi = (int)floorf(uf[l] + kTapSlack) - bmin + 1;
-      for (int b = lo; b <= hi; ++b) {
-        if (b >= 0 && b < nh)
-          atomicAdd(&hist[b], 1);
-        else
-          over = 1;
+      if (lo >= 0 && hi < nh) {  // lo, lo + 1 and, across a sample boundary, hi = lo + 2
+        atomicAdd(&hist[lo], 1);
+        atomicAdd(&hist[lo + 1], 1);
+        if (hi > lo + 1) atomicAdd(&hist[hi], 1);
+      } else {
+        over = 1;
       }
     }
     __syncwarp();
@@ -1062,14 +1151,21 @@ __global__ void __launch_bounds__(256) k_fwd_copies(unsigned long long* copies, 
     unsigned lo = 0, hi = 0;
 #pragma unroll
     for (int l = 0; l < 32; ++l) {
-      int best = 0;
-      unsigned best_sc = 0xffffffffu;
+      unsigned sc[kFwdCopies];
 #pragma unroll
-      for (int c = 0; c < kFwdCopies; ++c) {
-        const unsigned v = ld[(bins[l] + c * kFwdCopyRes) & 31];
-        const unsigned sc = __reduce_add_sync(0xffffffffu, v * v);
-        if (sc < best_sc) {
-          best_sc = sc;
+      for (int c = 0; c < kFwdCopies; c += 2) {
+        const unsigned v0 = ld[(bins[l] + c * kFwdCopyRes) & 31];
+        const unsigned v1 = ld[(bins[l] + (c + 1) * kFwdCopyRes) & 31];
+        const unsigned sum = __reduce_add_sync(0xffffffffu, v0 * v0 + ((v1 * v1) << 16));
+        sc[c] = sum & 0xffffu;
+        sc[c + 1] = sum >> 16;
+      }
+      int best = 0;
+      unsigned best_sc = sc[0];
+#pragma unroll
+      for (int c = 1; c < kFwdCopies; ++c) {
+        if (sc[c] < best_sc) {
+          best_sc = sc[c];
           best = c;
         }
       }

@@ -75,6 +75,8 @@ static pa_status build_table(pa_plan* p) {
                              kappa, p->t0 * p->fs, p->K, p->L, hmin, p->d_err, p->cap_stream));
   PA_CUDA(launch_fwd_copies(p->dim, p->d_fwd_copies, p->d_table, p->d_sensors, p->S, p->grid,
                             p->g, kappa, p->L, p->cap_stream));
+  PA_CUDA(launch_combine_order(p->d_table, p->d_sorted, p->d_upper, p->S, p->K, p->L, p->ntiles,
+                               p->cap_stream));
   int err = 0;
   PA_CUDA(cudaMemcpyAsync(&err, p->d_err, sizeof(int), cudaMemcpyDeviceToHost, p->cap_stream));
   PA_CUDA(cudaStreamSynchronize(p->cap_stream));
@@ -82,36 +84,6 @@ static pa_status build_table(pa_plan* p) {
     set_error("internal: a tile's arrival span exceeds the staged window (L=%d)", p->L);
     return PA_ERR_DEVICE_CHECK;
   }
-  // forward combine order: per sensor, the tiles that are not skipped sorted by
-  // window start (ties by tile index), and for every sample k the number of
-  // windows starting at or before k
-  const size_t n_tab = (size_t)p->ntiles * p->S;
-  std::vector<int> klo(n_tab);
-  PA_CUDA(cudaMemcpy2D(klo.data(), sizeof(int), p->d_table, sizeof(TileRef), sizeof(int), n_tab,
-                       cudaMemcpyDeviceToHost));
-  const int KL = p->K + p->L;
-  std::vector<int2> sorted(n_tab);
-  std::vector<int> upper((size_t)p->S * KL);
-  std::vector<int2> row;
-  for (int s = 0; s < p->S; ++s) {
-    row.clear();
-    for (int t = 0; t < p->ntiles; ++t) {
-      const int k0 = klo[(size_t)t * p->S + s];
-      if (k0 != kSkip) row.push_back(make_int2(t, window_start(k0)));
-    }
-    std::sort(row.begin(), row.end(), [](const int2& a, const int2& b) {
-      return a.y < b.y || (a.y == b.y && a.x < b.x);
-    });
-    std::copy(row.begin(), row.end(), sorted.begin() + (size_t)s * p->ntiles);
-    size_t i = 0;
-    for (int j = 0; j < KL; ++j) {
-      const int k = j - p->L;
-      while (i < row.size() && row[i].y <= k) ++i;
-      upper[(size_t)s * KL + j] = (int)i;
-    }
-  }
-  PA_CUDA(cudaMemcpy(p->d_sorted, sorted.data(), n_tab * sizeof(int2), cudaMemcpyHostToDevice));
-  PA_CUDA(cudaMemcpy(p->d_upper, upper.data(), upper.size() * sizeof(int), cudaMemcpyHostToDevice));
   return PA_OK;
 }
 
