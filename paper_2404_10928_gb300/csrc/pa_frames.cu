@@ -55,7 +55,7 @@ pa_status ensure_frames(pa_plan* p, int n) {
   const int old = p->frames_cap;
   const size_t N = (size_t)n_pix(p), SK = (size_t)n_trace(p);
   frame_free(p, &p->d_part_f, (size_t)old * p->S * p->ntiles * p->L);
-  frame_free(p, &p->d_packed_f, (size_t)old * p->S * p->Kp);
+  frame_free(p, &p->d_packed_f, (size_t)(old + (old & 1)) * p->S * p->Kp);
   frame_free(p, &p->d_parts_f, (size_t)old * p->n_partials);
   frame_free(p, &p->d_fsum, (size_t)2 * old);
   frame_free(p, &p->d_q_f, (size_t)old * SK);
@@ -63,14 +63,14 @@ pa_status ensure_frames(pa_plan* p, int n) {
   frame_free(p, &p->d_gz_f, (size_t)old * N);
   p->frames_cap = 0;
   PA_TRY(frame_alloc(p, &p->d_part_f, (size_t)n * p->S * p->ntiles * p->L));
-  PA_TRY(frame_alloc(p, &p->d_packed_f, (size_t)n * p->S * p->Kp));
+  PA_TRY(frame_alloc(p, &p->d_packed_f, (size_t)(n + (n & 1)) * p->S * p->Kp));  // frame pairs
   PA_TRY(frame_alloc(p, &p->d_parts_f, (size_t)n * p->n_partials));
   PA_TRY(frame_alloc(p, &p->d_fsum, (size_t)2 * n));
   PA_TRY(frame_alloc(p, &p->d_q_f, (size_t)n * SK));
   PA_TRY(frame_alloc(p, &p->d_r_f, (size_t)n * SK));
   PA_TRY(frame_alloc(p, &p->d_gz_f, (size_t)n * N));
   // the packed rows' zero padding stands for samples outside [0, K)
-  PA_CUDA(cudaMemset(p->d_packed_f, 0, (size_t)n * p->S * p->Kp * sizeof(float2)));
+  PA_CUDA(cudaMemset(p->d_packed_f, 0, (size_t)(n + (n & 1)) * p->S * p->Kp * sizeof(float2)));
   p->frames_cap = n;
   return PA_OK;
 }
@@ -109,40 +109,61 @@ pa_status fwd_frames(pa_plan* p, int n, const float* x, float* out, int mode, co
   return PA_OK;
 }
 
-// packs n frames of traces into the frames' packed rows
+// Packs n frames of traces: one frame into the plan's packed rows, several into
+// the frames' rows, interleaved by pairs (k_adjoint_frames).
 pa_status pack_frames(pa_plan* p, int n, const float* t, cudaStream_t st) {
-  PA_CUDA(launch_pack(t, p->d_packed_f, n * p->S, p->K, p->Kp, p->pad, st));
+  if (n == 1)
+    PA_CUDA(launch_pack(t, p->d_packed, p->S, p->K, p->Kp, p->pad, st));
+  else
+    PA_CUDA(launch_pack_frames(t, p->d_packed_f, p->S, p->K, p->Kp, p->pad, n, st));
   return PA_OK;
 }
 
-// A^T of the packed frames with the ADJ_AXPY epilogue
-pa_status adj_axpy_frames(pa_plan* p, int n, const float* xin, double coef, const float* tvg,
-                          double tvw, int nonneg, float* out, cudaStream_t st) {
-  AdjParams a = adjoint_params(p, out, ADJ_AXPY, nullptr, nonneg);
-  a.packed = p->d_packed_f;
-  a.xin = xin;
-  a.coef = (float)coef;
-  a.tvg = tvg;
-  a.tvw = (float)tvw;
+AdjParams frames_params(pa_plan* p, int n, float* out, int mode, int nonneg) {
+  AdjParams a = adjoint_params(p, out, mode, nullptr, nonneg);
+  if (n > 1) a.packed = p->d_packed_f;
   a.fs_img = n_pix(p);
-  a.fs_packed = (int64_t)p->S * p->Kp;
-  PA_CUDA(launch_adjoint(p->dim, a, p->cluster, p->ntiles, st, n));
-  return PA_OK;
+  return a;
+}
+
+void set_dc(pa_plan* p, AdjParams& a, const float* x, double scale, int accumulate, double* dc) {
+  a.dc_x = x;
+  a.red = make_reduce(p, OP_SUM, dc, nullptr, nullptr);
+  a.red.partials = p->d_parts_f;
+  a.red.post_scale = -scale * p->amp * p->fs / (p->c * p->c);  // d u / d c = -d fs / c^2
+  a.red.accumulate = accumulate;
 }
 
 // dc = (accumulate ? dc : 0) + scale * sum_f d/dc <g[f], A(x[f]; c)>, g packed
 pa_status dc_frames(pa_plan* p, int n, const float* x, double scale, int accumulate, double* dc,
                     cudaStream_t st) {
-  AdjParams a = adjoint_params(p, nullptr, ADJ_DC, nullptr, 0);
-  a.packed = p->d_packed_f;
+  AdjParams a = frames_params(p, n, nullptr, ADJ_DC, 0);
+  set_dc(p, a, x, scale, accumulate, dc);
   a.xin = x;
-  a.fs_img = n_pix(p);
-  a.fs_packed = (int64_t)p->S * p->Kp;
-  a.red = make_reduce(p, OP_SUM, dc, nullptr, nullptr);
-  a.red.partials = p->d_parts_f;
-  a.red.post_scale = -scale * p->amp * p->fs / (p->c * p->c);  // d u / d c = -d fs / c^2
-  a.red.accumulate = accumulate;
-  PA_CUDA(launch_adjoint(p->dim, a, p->cluster, p->ntiles, st, n));
+  PA_CUDA(n == 1 ? launch_adjoint(p->dim, a, p->cluster, p->ntiles, st)
+                 : launch_adjoint_frames(p->dim, a, p->cluster, p->ntiles, n, st));
+  return PA_OK;
+}
+
+// A^T of the packed frames with the ADJ_AXPY epilogue, and with dc != NULL the
+// dc_frames sum of the same packed traces against dc_x: one gather for both when
+// there are several frames
+pa_status adj_axpy_frames(pa_plan* p, int n, const float* xin, double coef, const float* tvg,
+                          double tvw, int nonneg, float* out, cudaStream_t st,
+                          const float* dc_x = nullptr, double dc_scale = 0.0, int dc_acc = 0,
+                          double* dc = nullptr) {
+  AdjParams a = frames_params(p, n, out, ADJ_AXPY, nonneg);
+  a.xin = xin;
+  a.coef = (float)coef;
+  a.tvg = tvg;
+  a.tvw = (float)tvw;
+  if (n == 1) {
+    if (dc) PA_TRY(dc_frames(p, n, dc_x, dc_scale, dc_acc, dc, st));
+    PA_CUDA(launch_adjoint(p->dim, a, p->cluster, p->ntiles, st));
+  } else {
+    if (dc) set_dc(p, a, dc_x, dc_scale, dc_acc, dc);
+    PA_CUDA(launch_adjoint_frames(p->dim, a, p->cluster, p->ntiles, n, st));
+  }
   return PA_OK;
 }
 
@@ -251,11 +272,9 @@ pa_status pa_tv_frames(pa_plan* plan, int n_frames, const float* x_dev, double e
   }
   Guard g(plan->device);
   cudaStream_t st = (cudaStream_t)stream;
-  const int64_t N = n_pix(plan);
-  for (int f = 0; f < n_frames; ++f)
-    PA_CUDA(launch_tv(plan->dim, x_dev + f * N, plan->grid.nx, plan->grid.ny, plan->grid.nz,
-                      (float)eps, grad_dev + f * N,
-                      make_reduce(plan, OP_SUM, tv_dev + f, nullptr, nullptr), st));
+  PA_CUDA(launch_tv_frames(plan->dim, x_dev, plan->grid.nx, plan->grid.ny, plan->grid.nz,
+                           (float)eps, grad_dev, n_frames,
+                           make_reduce(plan, OP_SUM, tv_dev, nullptr, nullptr), st));
   return PA_OK;
 }
 
@@ -297,16 +316,16 @@ pa_status pa_landweber_step_vjp_frames(pa_plan* plan, int n_frames, const float*
   PA_TRY(fwd_frames(plan, n_frames, gz, q, FWD_STORE, nullptr, st));
   if (gy_dev) PA_CUDA(launch_scale_by(gy_dev, q, (float)omega, SK, st));  // d/dy = omega A gz
   if (dc_dev) {
-    // d/dc = omega (<(dA/dc) gz, r> - <(dA/dc) x, A gz>) with r = y - A x
-    PA_TRY(pack_frames(plan, n_frames, q, st));
-    PA_TRY(dc_frames(plan, n_frames, x_dev, -omega, 0, dc_dev, st));
+    // d/dc = omega (<(dA/dc) gz, r> - <(dA/dc) x, A gz>) with r = y - A x; the
+    // second term comes with the gather of q below
     PA_TRY(fwd_frames(plan, n_frames, x_dev, plan->d_r_f, FWD_RESID, y_dev, st));
     PA_TRY(pack_frames(plan, n_frames, plan->d_r_f, st));
-    PA_TRY(dc_frames(plan, n_frames, gz, omega, 1, dc_dev, st));
+    PA_TRY(dc_frames(plan, n_frames, gz, omega, 0, dc_dev, st));
   }
   // d/dx = gz - omega A^T A gz
   PA_TRY(pack_frames(plan, n_frames, q, st));
-  return adj_axpy_frames(plan, n_frames, gz, -omega, nullptr, 0.0, 0, gx_dev, st);
+  return adj_axpy_frames(plan, n_frames, gz, -omega, nullptr, 0.0, 0, gx_dev, st, x_dev, -omega, 1,
+                         dc_dev);
 }
 
 pa_status pa_data_tv_loss_frames(pa_plan* plan, int n_frames, const float* x_dev,
@@ -327,13 +346,10 @@ pa_status pa_data_tv_loss_frames(pa_plan* plan, int n_frames, const float* x_dev
   double* tv = plan->d_fsum + n_frames;
   PA_TRY(fwd_frames(plan, n_frames, x_dev, r_dev, FWD_RESID, y_dev, st));
   PA_TRY(frame_sums(plan, n_frames, sq, st));
-  if (tv_weight != 0.0) {
-    const int64_t N = n_pix(plan);
-    for (int f = 0; f < n_frames; ++f)
-      PA_CUDA(launch_tv(plan->dim, x_dev + f * N, plan->grid.nx, plan->grid.ny, plan->grid.nz,
-                        (float)eps, tvgrad_dev + f * N,
-                        make_reduce(plan, OP_SUM, tv + f, nullptr, nullptr), st));
-  }
+  if (tv_weight != 0.0)
+    PA_CUDA(launch_tv_frames(plan->dim, x_dev, plan->grid.nx, plan->grid.ny, plan->grid.nz,
+                             (float)eps, tvgrad_dev, n_frames,
+                             make_reduce(plan, OP_SUM, tv, nullptr, nullptr), st));
   PA_CUDA(launch_affine_sum(sq, n_frames, tv, tv_weight != 0.0 ? n_frames : 0, tv_weight, loss_dev,
                             st));
   return PA_OK;
@@ -355,11 +371,12 @@ pa_status pa_data_tv_loss_vjp_frames(pa_plan* plan, int n_frames, const float* x
   // loss = sum_f ||y_f - A x_f||^2 + tv_weight TV(x_f), r = y - A x:
   // d/dx = -2 A^T r + tv_weight grad TV;  d/dc = -2 <r, (dA/dc) x>
   PA_TRY(pack_frames(plan, n_frames, r_dev, st));
-  if (dc_dev) PA_TRY(dc_frames(plan, n_frames, x_dev, -2.0 * g_loss, 0, dc_dev, st));
   if (gx_dev)
     PA_TRY(adj_axpy_frames(plan, n_frames, nullptr, -2.0 * g_loss,
                            tv_weight != 0.0 ? tvgrad_dev : nullptr, tv_weight * g_loss, 0, gx_dev,
-                           st));
+                           st, x_dev, -2.0 * g_loss, 0, dc_dev));
+  else
+    PA_TRY(dc_frames(plan, n_frames, x_dev, -2.0 * g_loss, 0, dc_dev, st));
   return PA_OK;
 }
 

@@ -167,11 +167,8 @@ struct AdjParams {
   const float* tvg;       // gradient of TV_eps at z (ADJ_FISTA), or the TV term (ADJ_AXPY)
   float l1, tv_beta, mu;
   float coef, tvw;        // ADJ_AXPY weights of A^T p and of tvg
-  // frames of one launch (blockIdx.z), all on the plan's geometry: strides
-  // between consecutive frames (0 for a single frame)
-  int64_t fs_img;         // out, xin, z, tvg: N
-  int64_t fs_packed;      // packed: S * Kp
-  int fs_red;             // OP_STORE partial slots per frame
+  const float* dc_x;      // launch_adjoint_frames: images weighting the slopes, or null
+  int64_t fs_img;         // launch_adjoint_frames: stride between frames' images, N
 };
 
 struct FwdParams {
@@ -301,8 +298,12 @@ cudaError_t launch_pack(const float* r, float2* packed, int S, int K, int Kp, in
                         cudaStream_t st);
 cudaError_t launch_bp_filter(const float* p, float2* packed, int S, int K, int Kp, int pad,
                              float t0fs, cudaStream_t st);
-cudaError_t launch_adjoint(int dim, const AdjParams& p, int cluster, int ntiles, cudaStream_t st,
-                           int frames = 1);
+cudaError_t launch_adjoint(int dim, const AdjParams& p, int cluster, int ntiles, cudaStream_t st);
+// several frames sharing their arrivals (k_adjoint_frames), packed by pairs
+cudaError_t launch_pack_frames(const float* r, float2* packed, int S, int K, int Kp, int pad,
+                               int frames, cudaStream_t st);
+cudaError_t launch_adjoint_frames(int dim, const AdjParams& p, int cluster, int ntiles, int frames,
+                                  cudaStream_t st);
 cudaError_t launch_forward(int dim, const FwdParams& p, cudaStream_t st, int frames = 1);
 int adjoint_smem_bytes(int L);
 cudaError_t configure_kernels(int smem_adj, int smem_fwd);
@@ -351,6 +352,8 @@ cudaError_t launch_fold_partials(float2* parts, int n, cudaStream_t st);
 cudaError_t launch_df_of(const double* v, float2* parts, cudaStream_t st);
 cudaError_t launch_tv(int dim, const float* x, int nx, int ny, int nz, float eps, float* grad,
                       const Reduce& red, cudaStream_t st);
+cudaError_t launch_tv_frames(int dim, const float* x, int nx, int ny, int nz, float eps, float* grad,
+                             int frames, const Reduce& red, cudaStream_t st);
 int tv_blocks(int64_t n);
 cudaError_t batch_kernel_config(int dim, size_t smem, int* blocks_per_sm);
 cudaError_t launch_batch_landweber(int dim, const BatchFrame* frames, int n_frames, const int* pre,

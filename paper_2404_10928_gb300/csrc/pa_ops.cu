@@ -935,14 +935,12 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint(const AdjParams P)
   const int rank = (int)cluster.block_rank();
   const int C = (int)cluster.num_blocks();
   const int tile = blockIdx.y;
-  const int frame = blockIdx.z;
   const int tid = threadIdx.x;
   const int s_begin = rank * P.sensors_per_rank;
   const int s_end = min(P.S, s_begin + P.sensors_per_rank);
-  float* s_acc = adj_accumulate<DIM, DC, NW>(P, P.packed + frame * P.fs_packed, tile,
-                                                    s_begin, s_end, smem);
-  float* out = P.out ? P.out + frame * P.fs_img : nullptr;
-  const float* xin = P.xin ? P.xin + frame * P.fs_img : nullptr;
+  float* s_acc = adj_accumulate<DIM, DC, NW>(P, P.packed, tile, s_begin, s_end, smem);
+  float* out = P.out;
+  const float* xin = P.xin;
 
   cluster.sync();
   // --------------- cluster reduction in rank order + epilogue ---------------
@@ -973,7 +971,7 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint(const AdjParams P)
         out[i] = xv;
       } else if (P.mode == ADJ_AXPY) {
         float xv = fmaf(P.coef, gval, xin ? xin[i] : 0.0f);
-        if (P.tvg) xv = fmaf(P.tvw, P.tvg[frame * P.fs_img + i], xv);
+        if (P.tvg) xv = fmaf(P.tvw, P.tvg[i], xv);
         if (P.nonneg) xv = fmaxf(xv, 0.0f);
         out[i] = xv;
       } else if (P.mode == ADJ_FISTA) {
@@ -1003,31 +1001,448 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint(const AdjParams P)
       if (rank == 0 && tid == 0) {
         DF u = df_zero();
         for (int q = 0; q < C; ++q) u = df_add(u, *cluster.map_shared_rank(&s_cta, q));
-        P.red.partials[frame * P.fs_red + tile] = make_float2(u.hi, u.lo);
+        P.red.partials[tile] = make_float2(u.hi, u.lo);
       }
     } else {
-      // one total over every frame of the launch
-      reduce_across_ctas<NW + 1>(P.red, t, (frame * gridDim.y + tile) * C + rank,
-                                        gridDim.x * gridDim.y * gridDim.z, s_red);
+      reduce_across_ctas<NW + 1>(P.red, t, tile * C + rank, gridDim.x * gridDim.y, s_red);
     }
   }
   cluster.sync();
   (void)TZ;
 }
 
-cudaError_t launch_adjoint(int dim, const AdjParams& p, int cluster, int ntiles, cudaStream_t st,
-                           int frames) {
+cudaError_t launch_adjoint(int dim, const AdjParams& p, int cluster, int ntiles, cudaStream_t st) {
   const bool dc = p.mode == ADJ_DC;
   if (p.warps == 4) {
     auto kernel = dim == 2 ? (dc ? k_adjoint<2, true, 4> : k_adjoint<2, false, 4>)
                            : (dc ? k_adjoint<3, true, 4> : k_adjoint<3, false, 4>);
-    return launch_k(kernel, dim3(cluster, ntiles, frames), dim3(32 * 5), adjoint_smem_bytes(p.L),
+    return launch_k(kernel, dim3(cluster, ntiles), dim3(32 * 5), adjoint_smem_bytes(p.L),
                     st, cluster, p);
   }
   auto kernel = dim == 2 ? (dc ? k_adjoint<2, true, kAdjWarps> : k_adjoint<2, false, kAdjWarps>)
                          : (dc ? k_adjoint<3, true, kAdjWarps> : k_adjoint<3, false, kAdjWarps>);
-  return launch_k(kernel, dim3(cluster, ntiles, frames), dim3(kAdjThreads), adjoint_smem_bytes(p.L),
+  return launch_k(kernel, dim3(cluster, ntiles), dim3(kAdjThreads), adjoint_smem_bytes(p.L),
                   st, cluster, p);
+}
+
+// ---------------------------------------------------------------------------
+// A^T (and the c-derivative's pixel sums) of several frames in one gather.
+//
+// Frames of a launch share the plan's geometry, so a pair's arrival and weight
+// are evaluated once and applied to 2 NP frames: their packed traces interleave
+// two frames per sample, (mid_0, mid_1, slope_0, slope_1), which one 16-byte
+// shared load and two (image) or one (slopes) packed instructions per sample
+// turn into both frames' terms.  MODE: ADJF_IMAGE, ADJF_SLOPES (the c-derivative) or
+// ADJF_BOTH, which takes both from the same loads.  Tiles, cluster split, sensor
+// order, the order of every sum and the slots of the partials are those of
+// k_adjoint over the same frames, so every result has the same bits.
+//
+// Per (pixel, sensor, frame) 10 thread instructions (ncu, 8 frames of 256^2, 128
+// sensors, prologue and epilogue included) against 17 + 15 for the image and the
+// slopes in two single-frame gathers: 67 + 76 -> 70 us for both there.  What
+// bounds it at that size is each CTA's start and end (16 sensors per CTA of an
+// 8-CTA cluster; 29% of the stalls are barriers); more stages, a reference
+// entry loaded a stage ahead and three CTAs per SM (72 registers) did not change it.
+// ---------------------------------------------------------------------------
+enum : int { ADJF_IMAGE = 0, ADJF_SLOPES = 1, ADJF_BOTH = 2 };
+
+// Pipeline: stages of 8 / NP sensors (eight frame-pair windows).  Four stages
+// while they leave room for two CTAs per SM, else two: a CTA has few sensors (16
+// of the 128 in an 8-CTA cluster), and with four stages all of its copies are in
+// flight at once.
+template <int NP> constexpr int kAdjfSB = 8 / NP;  // sensors per stage
+constexpr int kAdjfMaxStages = 4;
+__host__ __device__ inline int adjf_stages(int L) {
+  return 4 * 8 * L * (int)sizeof(float4) <= 80 * 1024 ? 4 : 2;
+}
+__host__ __device__ inline int adjf_planes(int mode, int np) { return 2 * np * (mode == ADJF_BOTH ? 2 : 1); }
+
+size_t adjoint_frames_smem(int L, int mode, int np) {
+  const size_t trace = (size_t)adjf_stages(L) * 8 * L * sizeof(float4);
+  const size_t acc = (size_t)adjf_planes(mode, np) * kTilePixels * sizeof(float);
+  return std::max(trace, acc) + kAdjfMaxStages * 8 * sizeof(TileRef2) +
+         2 * kAdjfMaxStages * sizeof(uint64_t);
+}
+
+__device__ __forceinline__ float4 lds_f4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+
+template <int DIM, bool NEAR, int MODE, int NP>
+__device__ __forceinline__ void adjf_pair2(const TileRef2& r, uint32_t base, uint32_t pstride,
+                                           float2 ddx, float2 ddy, float2 ddz, float2 cm,
+                                           float2 inv_kappa, float2 hik, float2 (&acc)[2][NP],
+                                           float2 (&accd)[2][NP], const Chk& chk) {
+  float2 rinv;
+  const float2 w = arrival2<DIM, NEAR>(r, ddx, ddy, ddz, cm, inv_kappa, hik, rinv);
+  const float2 t = add2(w, f2(kMagic));
+  const float2 e = fma2(add2(t, f2(-kMagic)), f2(-1.0f), w);  // w - n_c, in [-1/2, 1/2]
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {  // the two pixels
+    const float ti = i ? t.y : t.x, ei = i ? e.y : e.x, ri = i ? rinv.y : rinv.x;
+    const uint32_t a = base + ((uint32_t)__float_as_int(ti) << 4);
+#ifdef PA_CHECKED
+    const bool ok = chk_elem(chk, ti, chk.L - 1);
+#else
+    (void)chk;
+#endif
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+#ifdef PA_CHECKED
+      const float4 v = ok ? lds_f4(a + q * pstride) : make_float4(0.f, 0.f, 0.f, 0.f);
+#else
+      const float4 v = lds_f4(a + q * pstride);
+#endif
+      const float2 mid = make_float2(v.x, v.y), slope = make_float2(v.z, v.w);
+      if (MODE != ADJF_SLOPES) acc[i][q] = fma2(fma2(f2(ei), slope, mid), f2(ri), acc[i][q]);
+      if (MODE != ADJF_IMAGE) accd[i][q] = add2(accd[i][q], slope);
+    }
+  }
+}
+
+template <int DIM, int MODE, int NW, int NP>
+__global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint_frames(const AdjParams P, int frames) {
+  constexpr int NT = 32 * (NW + 1);
+  constexpr int NF = 2 * NP, NPL = MODE == ADJF_BOTH ? 2 * NF : NF;
+  constexpr int PPT = kTilePixels / (32 * NW), NPAIR = PPT / 2;
+  constexpr int SB = kAdjfSB<NP>;
+  constexpr int TX = Tile<DIM>::X, TY = Tile<DIM>::Y, TZ = Tile<DIM>::Z;
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ int s_abort, s_issued;
+  __shared__ DF s_red[NF][NW + 1];
+  __shared__ int s_last;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank(), C = (int)cluster.num_blocks();
+  const int tile = blockIdx.y, f0 = blockIdx.z * NF;
+  const int nf = min(NF, frames - f0);
+  const int L = P.L, NST = adjf_stages(L);
+  const int trace_bytes = max(NST * SB * NP * L * (int)sizeof(float4), NPL * kTilePixels * 4);
+  float4* s_trace = reinterpret_cast<float4*>(smem);
+  float* s_acc = reinterpret_cast<float*>(smem);  // the same memory once every window is read
+  TileRef2* s_ref = reinterpret_cast<TileRef2*>(smem + trace_bytes);
+  uint64_t* s_full = reinterpret_cast<uint64_t*>(s_ref + kAdjfMaxStages * 8);
+  uint64_t* s_empty = s_full + kAdjfMaxStages;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int s_begin = rank * P.sensors_per_rank;
+  const int s_end = min(P.S, s_begin + P.sensors_per_rank);
+  const int n_stages = s_end > s_begin ? (s_end - s_begin + SB - 1) / SB : 0;
+  if (tid == 0) {
+    for (int i = 0; i < NST; ++i) {
+      mbar_init(&s_full[i], 1);
+      mbar_init(&s_empty[i], NW);
+    }
+    s_abort = 0;
+    s_issued = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();
+
+  const int ttx = tile % P.g.ntx, tty = (tile / P.g.ntx) % P.g.nty, ttz = tile / (P.g.ntx * P.g.nty);
+  float2 acc[NPAIR][2][NP], accd[NPAIR][2][NP];
+  if (warp == NW) {
+    // ----------------------------- producer warp -----------------------------
+    // lane sb * NP + q copies frame pair q of sensor sb of the stage
+    const int sb = lane / NP, q = lane % NP;
+    auto entry = [&](int j) {  // the reference of this lane's sensor of stage j
+      const int s = s_begin + j * SB + sb;
+      TileRef r;
+      r.klo = kSkip;
+      if (sb < SB && s < s_end) r = P.table[(int64_t)tile * P.S + s];
+      return r;
+    };
+    int j = 0;
+    TileRef next = entry(0);
+    for (; j < n_stages; ++j) {
+      const int slot = j % NST;
+      TileRef r = next;
+      next = entry(j + 1);  // loaded a stage ahead
+      if (j >= NST) {
+        int ok = 1;
+        if (lane == 0) ok = mbar_wait_bounded(&s_empty[slot], ((j / NST) - 1) & 1);
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) {
+          if (lane == 0) {
+            atomicOr(P.err, ERR_WAIT_TIMEOUT);
+            s_abort = 1;
+          }
+          break;
+        }
+      }
+      const int s = s_begin + j * SB + sb;
+      uint32_t bytes = 0;
+      const float4* src = nullptr;
+      if (sb < SB) {
+        if (r.klo != kSkip) {
+          const int ws0 = P.pad + window_start(r.klo);
+#ifdef PA_CHECKED
+          if (ws0 < 0 || ws0 + L > P.Kp) {  // the window must lie inside its packed row
+            atomicOr(P.err, ERR_INDEX);
+            r.klo = kSkip;
+          } else
+#endif
+          if (2 * q < nf) {
+            bytes = (uint32_t)L * (uint32_t)sizeof(float4);
+            src = reinterpret_cast<const float4*>(P.packed) +
+                  ((int64_t)(f0 / 2 + q) * P.S + s) * P.Kp + ws0;
+          }
+        }
+        if (q == 0) {
+          if (r.klo != kSkip)
+            s_ref[slot * 8 + sb] = expand_ref(r);
+          else
+            s_ref[slot * 8 + sb].klo = kSkip;
+        }
+      }
+      const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+      __syncwarp();
+      if (lane == 0) mbar_arrive_expect_tx(&s_full[slot], total);
+      __syncwarp();
+      if (bytes) bulk_g2s(s_trace + ((slot * SB + sb) * NP + q) * L, src, bytes, &s_full[slot]);
+    }
+    if (lane == 0) s_issued = j;
+  } else {
+    // ----------------------------- compute warps -----------------------------
+    float2 ddx[NPAIR], ddy[NPAIR], ddz[NPAIR], cm[NPAIR];
+    int nvx, nvy, nvz;
+    tile_valid<DIM>(ttx, tty, ttz, P.g, nvx, nvy, nvz);
+#pragma unroll
+    for (int m = 0; m < PPT; ++m) {
+      int lx, ly, lz;
+      float ox, oy, oz, oc;
+      pixel_local<DIM>(tid + m * 32 * NW, lx, ly, lz);
+      clamp_local<DIM>(ttx, tty, ttz, P.g, lx, ly, lz);
+      pixel_offset<DIM>(lx, ly, lz, nvx, nvy, nvz, P.g, P.kappa, ox, oy, oz, oc);
+      set_lane(ddx[m >> 1], m & 1, ox);
+      set_lane(ddy[m >> 1], m & 1, oy);
+      set_lane(ddz[m >> 1], m & 1, oz);
+      set_lane(cm[m >> 1], m & 1, oc);
+#pragma unroll
+      for (int q = 0; q < NP; ++q) acc[m >> 1][m & 1][q] = accd[m >> 1][m & 1][q] = f2(0.0f);
+    }
+    const float2 inv_kappa = f2(P.inv_kappa), hik = f2(P.half_inv_kappa);
+    const Chk chk{L, P.err};
+    const uint32_t trace_u32 = smem_u32(s_trace), pstride = 16u * (uint32_t)L;
+    for (int j = 0; j < n_stages; ++j) {
+      const int slot = j % NST;
+      const bool ok = mbar_wait_bounded(&s_full[slot], (j / NST) & 1);
+      if (__any_sync(0xffffffffu, !ok)) {
+        if (lane == 0) {
+          atomicOr(P.err, ERR_WAIT_TIMEOUT);
+          s_abort = 1;
+        }
+        break;
+      }
+      if (*(volatile int*)&s_abort) break;
+      const TileRef2* refs = s_ref + slot * 8;
+      uint32_t base = magic_base(trace_u32 + (uint32_t)(slot * SB * NP * L + L / 2) * 16u, 4);
+#pragma unroll 1
+      for (int sb = 0; sb < SB; ++sb, base += NP * pstride) {
+        const TileRef2 r = refs[sb];
+        if (r.klo == kSkip) continue;
+        if (r.klo & kNear) {
+#pragma unroll
+          for (int h = 0; h < NPAIR; ++h)
+            adjf_pair2<DIM, true, MODE, NP>(r, base, pstride, ddx[h], ddy[h], ddz[h], cm[h],
+                                            inv_kappa, hik, acc[h], accd[h], chk);
+        } else {
+#pragma unroll
+          for (int h = 0; h < NPAIR; ++h)
+            adjf_pair2<DIM, false, MODE, NP>(r, base, pstride, ddx[h], ddy[h], ddz[h], cm[h],
+                                             inv_kappa, hik, acc[h], accd[h], chk);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&s_empty[slot]);
+    }
+  }
+  __syncthreads();
+  if (s_abort) {
+    // drain copies that may still be in flight before the memory is reused (bounded)
+    if (tid == 0) {
+      const int issued = s_issued;
+      for (int jj = max(0, issued - NST); jj < issued; ++jj)
+        mbar_wait_bounded(&s_full[jj % NST], (jj / NST) & 1);
+    }
+    __syncthreads();
+  }
+  // planes 0..NF-1: images (or slopes alone), NF..: slopes
+  if (warp < NW) {
+#pragma unroll
+    for (int m = 0; m < PPT; ++m) {
+      int lx, ly, lz;
+      pixel_local<DIM>(tid + m * 32 * NW, lx, ly, lz);
+      float* a = s_acc + rowmajor_index<DIM>(lx, ly, lz);
+#pragma unroll
+      for (int q = 0; q < NP; ++q) {
+        const float2 v = MODE == ADJF_SLOPES ? accd[m >> 1][m & 1][q] : acc[m >> 1][m & 1][q];
+        a[(2 * q) * kTilePixels] = v.x;
+        a[(2 * q + 1) * kTilePixels] = v.y;
+        if (MODE == ADJF_BOTH) {
+          const float2 d = accd[m >> 1][m & 1][q];
+          a[(NF + 2 * q) * kTilePixels] = d.x;
+          a[(NF + 2 * q + 1) * kTilePixels] = d.y;
+        }
+      }
+    }
+  }
+  cluster.sync();
+  // --------------- cluster reduction in rank order + epilogue ---------------
+  const int per = (kTilePixels + C - 1) / C;
+  const int p0 = rank * per, p1 = min(kTilePixels, p0 + per);
+  // warps in groups of four (128 pixels), group w / 4 taking frames w / 4, w / 4 +
+  // kGroups, ...: the frames' remote loads are in flight together.  A frame's
+  // partial keeps the order of k_adjoint's block of NT threads (thread p - p0 mod
+  // NT, warps in order, a warp without pixels adding nothing): with C = 8 a group's
+  // four warps are those with pixels; otherwise one thread block per frame in turn.
+  constexpr int kGroups = NW / 4;
+  const bool grouped = per == 128;
+  DF part[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) part[f] = df_zero();
+  auto sum = [&](int plane, int p) {  // the C <= 8 remote loads together, summed in rank order
+    float pq[8], v = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      pq[q] = q < C ? cluster.map_shared_rank(s_acc, q)[plane * kTilePixels + p] : 0.0f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (q < C) v += pq[q];
+    return v;
+  };
+  const int grp = warp >> 2;
+  for (int p = p0 + (grouped ? tid & 127 : tid); p < p1 && !(grouped && grp >= kGroups);
+       p += grouped ? 128 : NT) {
+    int lx, ly, lz;
+    pixel_rowmajor<DIM>(p, lx, ly, lz);
+    const int gx = ttx * TX + lx, gy = tty * TY + ly, gz = ttz * TZ + lz;
+    if (gx >= P.g.nx || gy >= P.g.ny || gz >= P.g.nz) continue;
+    const int64_t i0 = ((int64_t)gz * P.g.ny + gy) * P.g.nx + gx;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      if (f >= nf || (grouped && f % kGroups != grp)) continue;
+      const int64_t i = (f0 + f) * P.fs_img + i0;
+      if (MODE != ADJF_IMAGE)  // before the image is stored, which may replace x
+        part[f] = df_add(part[f], df_prod(P.dc_x[i], sum(MODE == ADJF_BOTH ? NF + f : f, p)));
+      if (MODE != ADJF_SLOPES) {
+        const float gval = P.amp * sum(f, p);
+        float xv = fmaf(P.coef, gval, P.xin ? P.xin[i] : 0.0f);
+        if (P.tvg) xv = fmaf(P.tvw, P.tvg[i], xv);
+        if (P.nonneg) xv = fmaxf(xv, 0.0f);
+        P.out[i] = xv;
+      }
+    }
+  }
+  if (MODE != ADJF_IMAGE) {
+    // one partial per (frame, tile, rank), in the slots of a launch with one
+    // frame per CTA; the last CTA sums them
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) part[f] = df_add(part[f], df_shfl_xor(part[f], o));
+      if (lane == 0) s_red[f][warp] = part[f];
+    }
+    __syncthreads();
+    if (tid < nf) {
+      DF u = df_zero();
+      const int w0 = grouped ? 4 * (tid % kGroups) : 0, w1 = grouped ? w0 + 4 : NW + 1;
+      for (int w = w0; w < w1; ++w) u = df_add(u, s_red[tid][w]);
+      P.red.partials[((f0 + tid) * gridDim.y + tile) * C + rank] = make_float2(u.hi, u.lo);
+      __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0)
+      s_last = atomicAdd(P.red.counter, 1u) == gridDim.x * gridDim.y * gridDim.z - 1u;
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      const int nblk = frames * gridDim.y * C;
+      DF v = df_zero();
+      for (int i = tid; i < nblk; i += NT) {
+        const float2 w = __ldcg(P.red.partials + i);
+        v = df_add(v, DF{w.x, w.y});
+      }
+      const DF total = block_sum<NW + 1>(v, s_red[0]);
+      if (tid == 0) {
+        const double d = df_to_double(total) * P.red.post_scale;
+        *P.red.out_sum = P.red.accumulate ? *P.red.out_sum + d : d;
+        *P.red.counter = 0u;
+      }
+    }
+  }
+  cluster.sync();
+}
+
+// Interleaved packing of frame pairs: row (pair, sensor) of Kp (mid_0, mid_1,
+// slope_0, slope_1); an odd last frame is its own partner (the second result is
+// not stored).
+__global__ void k_pack_frames(const float* r, float4* packed, int S, int K, int Kp, int pad,
+                              int frames) {
+  const int s = blockIdx.y, pair = blockIdx.z;
+  const int k4 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (k4 > K) return;  // entries k in [-1, K)
+  const float* r0 = r + ((int64_t)(2 * pair) * S + s) * K;
+  const float* r1 = 2 * pair + 1 < frames ? r0 + (int64_t)S * K : r0;
+  float4* row = packed + ((int64_t)pair * S + s) * Kp + pad;
+  float v[2][5];
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    const int k = k4 - 1 + j;  // r_{-1} = r_K = 0
+    const bool in = k >= 0 && k < K;
+    v[0][j] = in ? r0[k] : 0.0f;
+    v[1][j] = in ? r1[k] : 0.0f;
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int k = k4 - 1 + j;
+    if (k < K)
+      row[k] = make_float4(0.5f * (v[0][j] + v[0][j + 1]), 0.5f * (v[1][j] + v[1][j + 1]),
+                           v[0][j + 1] - v[0][j], v[1][j + 1] - v[1][j]);
+  }
+}
+
+cudaError_t launch_pack_frames(const float* r, float2* packed, int S, int K, int Kp, int pad,
+                               int frames, cudaStream_t st) {
+  const int threads = 128;
+  const dim3 grid((K + 1 + 4 * threads - 1) / (4 * threads), S, (frames + 1) / 2);
+  return launch_k(k_pack_frames, grid, dim3(threads), 0, st, 0, r, reinterpret_cast<float4*>(packed),
+                  S, K, Kp, pad, frames);
+}
+
+using AdjFramesKernel = void (*)(const AdjParams, int);
+template <int D, int W, int N>
+AdjFramesKernel adjoint_frames_kernel(int mode) {
+  return mode == ADJF_IMAGE    ? k_adjoint_frames<D, ADJF_IMAGE, W, N>
+         : mode == ADJF_SLOPES ? k_adjoint_frames<D, ADJF_SLOPES, W, N>
+                               : k_adjoint_frames<D, ADJF_BOTH, W, N>;
+}
+AdjFramesKernel adjoint_frames_kernel(int dim, int mode, int warps, int np) {
+  if (dim == 2)
+    return warps == 4 ? (np == 2 ? adjoint_frames_kernel<2, 4, 2>(mode)
+                                 : adjoint_frames_kernel<2, 4, 1>(mode))
+                      : (np == 2 ? adjoint_frames_kernel<2, kAdjWarps, 2>(mode)
+                                 : adjoint_frames_kernel<2, kAdjWarps, 1>(mode));
+  return warps == 4 ? (np == 2 ? adjoint_frames_kernel<3, 4, 2>(mode)
+                               : adjoint_frames_kernel<3, 4, 1>(mode))
+                    : (np == 2 ? adjoint_frames_kernel<3, kAdjWarps, 2>(mode)
+                               : adjoint_frames_kernel<3, kAdjWarps, 1>(mode));
+}
+
+// mode ADJ_AXPY (the image), ADJ_DC (the slopes against dc_x), or ADJ_AXPY with
+// dc_x set (both); frames >= 2
+cudaError_t launch_adjoint_frames(int dim, const AdjParams& p, int cluster, int ntiles, int frames,
+                                  cudaStream_t st) {
+  const int mode = p.mode == ADJ_DC ? ADJF_SLOPES : p.dc_x ? ADJF_BOTH : ADJF_IMAGE;
+  const int np = frames > 2 ? 2 : 1;
+  const AdjFramesKernel kernel = adjoint_frames_kernel(dim, mode, p.warps, np);
+  const size_t smem = adjoint_frames_smem(p.L, mode, np);
+  const int threads = 32 * ((p.warps == 4 ? 4 : kAdjWarps) + 1);
+  return launch_k(kernel, dim3(cluster, ntiles, (frames + 2 * np - 1) / (2 * np)), dim3(threads),
+                  smem, st, cluster, p, frames);
 }
 
 // ---------------------------------------------------------------------------
@@ -1570,6 +1985,17 @@ cudaError_t configure_kernels(int smem_adj, int smem_fwd) {
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_adj)) !=
         cudaSuccess)
       return e;
+  // the frames' gathers take at most the single-frame gather's windows, or 80 KB of
+  // stages (adjf_stages)
+  const int smem_frames = std::max(smem_adj, 88 * 1024);
+  for (int dim = 2; dim <= 3; ++dim)
+    for (int mode = ADJF_IMAGE; mode <= ADJF_BOTH; ++mode)
+      for (int warps = 4; warps <= 8; warps += 4)
+        for (int np = 1; np <= 2; ++np)
+          if ((e = cudaFuncSetAttribute(adjoint_frames_kernel(dim, mode, warps, np),
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        smem_frames)) != cudaSuccess)
+            return e;
   const void* fwd[] = {
       (const void*)k_fwd_tile<2, false, 64>,  (const void*)k_fwd_tile<2, true, 64>,
       (const void*)k_fwd_tile<3, false, 64>,  (const void*)k_fwd_tile<3, true, 64>,
@@ -1925,7 +2351,9 @@ cudaError_t launch_norm(const float* v, int64_t n, const Reduce& red, int nblk, 
 // the last index (Neumann).  One thread per pixel writes the gradient
 //   dTV/dx_i = -sum_a a_a(i) + sum_a a_a(i - e_a),  a_a = (forward diff along a)/m,
 // recomputing its neighbours' terms (no inter-thread exchange); the value is
-// reduced in FP64 inside the kernel.
+// reduced in double-float inside the kernel.  Several images (frames) take one
+// launch, frame blockIdx.y with its share of the partials, and the last CTA sums
+// every frame's (eight 256^2 frames: 8 launches of 7.7 us -> one of 13 us).
 // ---------------------------------------------------------------------------
 template <int DIM>
 __device__ __forceinline__ void tv_terms(const float* x, int i, int j, int l, int nx,
@@ -1944,12 +2372,14 @@ __device__ __forceinline__ void tv_terms(const float* x, int i, int j, int l, in
 }
 
 template <int DIM>
-__global__ void __launch_bounds__(kVecThreads) k_tv(const float* x, int nx, int ny,
-                                                    int nz, float eps, float* grad,
+__global__ void __launch_bounds__(kVecThreads) k_tv(const float* images, int nx, int ny,
+                                                    int nz, float eps, float* grads,
                                                     const Reduce red) {
   __shared__ DF s_red[kVecThreads / 32];
   const float eps2 = eps * eps;
   const int64_t n = (int64_t)nx * ny * nz;
+  const float* x = images + blockIdx.y * n;
+  float* grad = grads + blockIdx.y * n;
   DF part = df_zero();
   for (int64_t o = blockIdx.x * (int64_t)kVecThreads + threadIdx.x; o < n;
        o += (int64_t)gridDim.x * kVecThreads) {
@@ -1974,7 +2404,24 @@ __global__ void __launch_bounds__(kVecThreads) k_tv(const float* x, int nx, int 
     grad[o] = g;
   }
   const DF t = block_sum<kVecThreads / 32>(part, s_red);
-  reduce_across_ctas<kVecThreads / 32>(red, t, blockIdx.x, gridDim.x, s_red);
+  if (gridDim.y == 1) {
+    reduce_across_ctas<kVecThreads / 32>(red, t, blockIdx.x, gridDim.x, s_red);
+    return;
+  }
+  __shared__ int s_last;
+  if (threadIdx.x == 0) {
+    red.partials[blockIdx.y * gridDim.x + blockIdx.x] = make_float2(t.hi, t.lo);
+    __threadfence();
+    s_last = atomicAdd(red.counter, 1u) == gridDim.x * gridDim.y - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int f = threadIdx.x >> 5; f < (int)gridDim.y; f += kVecThreads / 32) {
+    const DF u = warp_sum_partials(red.partials + f * gridDim.x, gridDim.x);
+    if ((threadIdx.x & 31) == 0) red.out_sum[f] = df_to_double(u);
+  }
+  if (threadIdx.x == 0) *red.counter = 0u;
 }
 
 int tv_blocks(int64_t n) {
@@ -1986,6 +2433,23 @@ cudaError_t launch_tv(int dim, const float* x, int nx, int ny, int nz, float eps
   const int nb = tv_blocks((int64_t)nx * ny * nz);
   return launch_k(dim == 2 ? k_tv<2> : k_tv<3>, dim3(nb), dim3(kVecThreads), 0, st, 0, x, nx, ny,
                   nz, eps, grad, red);
+}
+
+// Frames share the plan's 152 * 8 partials: groups of at most that many frames.
+cudaError_t launch_tv_frames(int dim, const float* x, int nx, int ny, int nz, float eps, float* grad,
+                             int frames, const Reduce& red, cudaStream_t st) {
+  const int64_t n = (int64_t)nx * ny * nz;
+  constexpr int kSlots = 152 * 8;
+  for (int f0 = 0; f0 < frames; f0 += kSlots) {
+    const int nf = std::min(kSlots, frames - f0);
+    const int nb = nf == 1 ? tv_blocks(n) : std::min(tv_blocks(n), kSlots / nf);
+    Reduce r = red;
+    r.out_sum = red.out_sum + f0;
+    const cudaError_t e = launch_k(dim == 2 ? k_tv<2> : k_tv<3>, dim3(nb, nf), dim3(kVecThreads), 0,
+                                   st, 0, x + f0 * n, nx, ny, nz, eps, grad + f0 * n, r);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 
