@@ -348,7 +348,7 @@ class Plan:
                 raise ValueError(f"{name} must hold {n} frames")
         gx = torch.empty((n, self.n_pixels), device=self.device)
         gy = torch.empty((n, self.n_sensors, self.n_samples), device=self.device) if need_y else None
-        gc = torch.zeros((), dtype=torch.float64, device=self.device) if need_c else None
+        gc = torch.empty((), dtype=torch.float64, device=self.device) if need_c else None
         check(self._lib.pa_landweber_step_vjp_frames(
             self._h, n, x.data_ptr(), y.data_ptr(), x_out.data_ptr(), g_out.data_ptr(),
             float(omega), int(bool(nonneg)), gx.data_ptr(),
@@ -376,7 +376,7 @@ class Plan:
         n = self._frames_img(x, "x")
         self._frames_trace(r, n, "r")
         gx = torch.empty((n, self.n_pixels), device=self.device) if need_x else None
-        gc = torch.zeros((), dtype=torch.float64, device=self.device) if need_c else None
+        gc = torch.empty((), dtype=torch.float64, device=self.device) if need_c else None
         check(self._lib.pa_data_tv_loss_vjp_frames(
             self._h, n, x.data_ptr(), r.data_ptr(),
             tvgrad.data_ptr() if tvgrad is not None else None, float(tv_weight), float(g_loss),

@@ -23,7 +23,10 @@ dimensions are frames sharing the plan's geometry and c).
   is recomputed in backward).
 
 c is a 0-d tensor; changing it rebuilds the plan's reference table (a
-blocking call).
+blocking call).  Reading its value waits for the device when c lives there, so
+each forward pass reads it once (the unrolled loop once for all its steps) and
+the backward pass uses the value read: 12 reads -> 1 in a pass of four unrolled
+steps with its backward, each of which had left the device idle for 30-80 us.
 """
 from __future__ import annotations
 
@@ -31,8 +34,11 @@ import torch
 from torch.utils.checkpoint import checkpoint
 
 
-def _set_c(plan, c) -> None:
-    cv = float(c)
+def _value(c) -> float:
+    return float(c.detach())
+
+
+def _set_c(plan, cv: float) -> None:
     if cv != plan.c:
         plan.set_sound_speed(cv)
 
@@ -56,7 +62,8 @@ class ForwardOp(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, c, plan):
-        _set_c(plan, c)
+        ctx.cv = _value(c)
+        _set_c(plan, ctx.cv)
         xb = _img(x, plan)
         out = plan.forward_frames(xb)
         ctx.plan = plan
@@ -68,7 +75,7 @@ class ForwardOp(torch.autograd.Function):
     def backward(ctx, gp):
         xb, c = ctx.saved_tensors
         plan = ctx.plan
-        _set_c(plan, c)
+        _set_c(plan, ctx.cv)
         gb = _trace(gp.to(torch.float32), plan)
         gx = gc = None
         if ctx.needs_input_grad[0]:
@@ -83,7 +90,8 @@ class AdjointOp(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, r, c, plan):
-        _set_c(plan, c)
+        ctx.cv = _value(c)
+        _set_c(plan, ctx.cv)
         rb = _trace(r, plan)
         out = plan.adjoint_frames(rb)
         ctx.plan = plan
@@ -95,7 +103,7 @@ class AdjointOp(torch.autograd.Function):
     def backward(ctx, gg):
         rb, c = ctx.saved_tensors
         plan = ctx.plan
-        _set_c(plan, c)
+        _set_c(plan, ctx.cv)
         gb = _img(gg.to(torch.float32), plan)
         gr = gc = None
         if ctx.needs_input_grad[0]:
@@ -129,7 +137,8 @@ class DataTVLoss(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, c, p, plan, tv_weight, eps):
-        _set_c(plan, c)
+        ctx.cv = _value(c)
+        _set_c(plan, ctx.cv)
         xb = _img(x, plan)
         loss, r, tg = plan.data_tv_loss_frames(xb, _trace(p.to(torch.float32), plan),
                                                float(tv_weight), float(eps))
@@ -144,7 +153,7 @@ class DataTVLoss(torch.autograd.Function):
     def backward(ctx, g):
         xb, r, tg, c = ctx.saved_tensors
         plan = ctx.plan
-        _set_c(plan, c)
+        _set_c(plan, ctx.cv)
         gx, gc = plan.data_tv_loss_vjp_frames(xb, r, tg if ctx.has_tv else None, ctx.tv_weight,
                                               _upstream(g), need_x=ctx.needs_input_grad[0],
                                               need_c=ctx.needs_input_grad[1])
@@ -162,11 +171,13 @@ def data_tv_loss(plan, x, c, p, tv_weight: float = 1e-3, eps: float = 1e-4):
 
 class LandweberStep(torch.autograd.Function):
     """x_out = max(0, x + omega A^T (y - A(x; c))) (the projection only with
-    nonneg), with gradients in x, y and c."""
+    nonneg), with gradients in x, y and c.  cv: the value of c when the caller
+    has read it."""
 
     @staticmethod
-    def forward(ctx, x, y, c, plan, omega, nonneg):
-        _set_c(plan, c)
+    def forward(ctx, x, y, c, plan, omega, nonneg, cv=None):
+        ctx.cv = _value(c) if cv is None else cv
+        _set_c(plan, ctx.cv)
         xb = _img(x, plan)
         yb = _trace(y, plan)
         out = plan.landweber_step_frames(xb, yb, float(omega), bool(nonneg))
@@ -180,7 +191,7 @@ class LandweberStep(torch.autograd.Function):
     def backward(ctx, g):
         xb, yb, out, c = ctx.saved_tensors
         plan = ctx.plan
-        _set_c(plan, c)
+        _set_c(plan, ctx.cv)
         gx, gy, gc = plan.landweber_step_vjp_frames(
             xb, yb, out, _img(g.to(torch.float32), plan), ctx.omega, ctx.nonneg,
             need_y=ctx.needs_input_grad[1], need_c=ctx.needs_input_grad[2])
@@ -189,7 +200,7 @@ class LandweberStep(torch.autograd.Function):
             gy = gy.reshape(ctx.shapes[1])
         if gc is not None:
             gc = gc.to(c.dtype)
-        return gx, gy, gc, None, None, None
+        return gx, gy, gc, None, None, None, None
 
 
 class UnrolledLandweber(torch.nn.Module):
@@ -206,14 +217,19 @@ class UnrolledLandweber(torch.nn.Module):
         self.checkpointing = checkpointing
         self.nonneg = bool(nonneg)
 
-    def step(self, x, y, c):
-        return LandweberStep.apply(x, y, c, self.plan, self.omega, self.nonneg)
+    def step(self, x, y, c, cv=None):
+        return LandweberStep.apply(x, y, c, self.plan, self.omega, self.nonneg, cv)
 
     def forward(self, x0, y, c):
         x = x0
+        # an overridden step takes (x, y, c) and may draw random numbers; the
+        # class's own takes the value of c, read once, and draws none
+        own = type(self).step is UnrolledLandweber.step
+        args = (y, c, _value(c)) if own else (y, c)
         for _ in range(self.n_iter):
             if self.checkpointing:
-                x = checkpoint(self.step, x, y, c, use_reentrant=False)
+                x = checkpoint(self.step, x, *args, use_reentrant=False,
+                               preserve_rng_state=not own)
             else:
-                x = self.step(x, y, c)
+                x = self.step(x, *args)
         return x
