@@ -83,13 +83,15 @@ typedef struct {
  *   y_dtype     storage type of the measured traces y passed to pa_reconstruct
  *               (PA_F32 or PA_F16; the arithmetic stays FP32).
  *   adj_cluster CTAs that split one pixel tile's sensors in the adjoint (1, 2, 4
- *               or 8; 0 = chosen from the grid size).  Results are identical up
+ *               or 8; 0 = chosen from the grid and sensor count).  Results are identical up
  *               to the order of the final per-pixel sum.
- *   fwd_sensors_per_cta  sensors per forward-gather work item (1..256; 0 = 32).
+ *   fwd_sensors_per_cta  sensors per forward-gather work item (1..256; 0 = chosen
+ *               from the grid and sensor count).
  *   fwd_threads  threads per forward-gather CTA: 64, 128 or 256, each owning
  *               1024 / fwd_threads pixels of the tile (0 = 128).
  *   adj_warps    compute warps per adjoint CTA: 4 or 8, each thread owning
- *               1024 / (32 adj_warps) pixels of the tile (0 = 8).
+ *               1024 / (32 adj_warps) pixels of the tile (0 = chosen from the
+ *               dimension and adj_cluster).
  * The last four are the tile shapes an autotuner may pick; none changes a
  * result bit of the forward (its window sums are exact integer sums), and
  * adj_warps none of the adjoint's image (each pixel sums its sensors in

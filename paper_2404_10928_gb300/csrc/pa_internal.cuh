@@ -275,7 +275,7 @@ constexpr int kAdjStages = 4;
 // forward kernel shape
 constexpr int kFwdThreads = 256;             // fwd_tile_block's default pixel owners (4 pixels each)
 constexpr int kFwdThreadsDefault = 128;      // k_fwd_tile's default block (8 pixels per thread)
-constexpr int kFwdSPC = 32;                  // default sensors per tile work item
+constexpr int kFwdSPC = 32;                  // sensors per tile work item that every plan can hold
 // sensors per accumulation stage of the forward: 8 in 2D, 4 in 3D (there the
 // gather is bound by shared memory, and smaller window buffers fit more CTAs
 // per SM: the 128^3 forward 2.09 against 2.17 ms; 2D is 0.5% faster with 8)
@@ -315,6 +315,9 @@ __host__ __device__ inline int combine_kblocks(int K, int threads, int spt) {
   return (K + spt * threads - 1) / (spt * threads);
 }
 pa_status validate_grid(const pa_grid* g);
+// the adjoint's work split where the caller leaves it open (pa_plan.cu)
+int default_cluster(int dim, int64_t ntiles, int S, int sms);
+int default_adj_warps(int dim, int cluster);
 
 // reductions and vector updates
 cudaError_t launch_cgls_xr(float* x, const float* pvec, const float* r_in, float* r_out,

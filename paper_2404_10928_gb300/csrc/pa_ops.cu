@@ -1420,16 +1420,12 @@ AdjFramesKernel adjoint_frames_kernel(int mode) {
          : mode == ADJF_SLOPES ? k_adjoint_frames<D, ADJF_SLOPES, W, N>
                                : k_adjoint_frames<D, ADJF_BOTH, W, N>;
 }
-AdjFramesKernel adjoint_frames_kernel(int dim, int mode, int warps, int np) {
+AdjFramesKernel adjoint_frames_kernel(int dim, int mode, int np) {
   if (dim == 2)
-    return warps == 4 ? (np == 2 ? adjoint_frames_kernel<2, 4, 2>(mode)
-                                 : adjoint_frames_kernel<2, 4, 1>(mode))
-                      : (np == 2 ? adjoint_frames_kernel<2, kAdjWarps, 2>(mode)
-                                 : adjoint_frames_kernel<2, kAdjWarps, 1>(mode));
-  return warps == 4 ? (np == 2 ? adjoint_frames_kernel<3, 4, 2>(mode)
-                               : adjoint_frames_kernel<3, 4, 1>(mode))
-                    : (np == 2 ? adjoint_frames_kernel<3, kAdjWarps, 2>(mode)
-                               : adjoint_frames_kernel<3, kAdjWarps, 1>(mode));
+    return np == 2 ? adjoint_frames_kernel<2, kAdjWarps, 2>(mode)
+                   : adjoint_frames_kernel<2, kAdjWarps, 1>(mode);
+  return np == 2 ? adjoint_frames_kernel<3, kAdjWarps, 2>(mode)
+                 : adjoint_frames_kernel<3, kAdjWarps, 1>(mode);
 }
 
 // mode ADJ_AXPY (the image), ADJ_DC (the slopes against dc_x), or ADJ_AXPY with
@@ -1438,11 +1434,12 @@ cudaError_t launch_adjoint_frames(int dim, const AdjParams& p, int cluster, int 
                                   cudaStream_t st) {
   const int mode = p.mode == ADJ_DC ? ADJF_SLOPES : p.dc_x ? ADJF_BOTH : ADJF_IMAGE;
   const int np = frames > 2 ? 2 : 1;
-  const AdjFramesKernel kernel = adjoint_frames_kernel(dim, mode, p.warps, np);
+  const AdjFramesKernel kernel = adjoint_frames_kernel(dim, mode, np);
   const size_t smem = adjoint_frames_smem(p.L, mode, np);
-  const int threads = 32 * ((p.warps == 4 ? 4 : kAdjWarps) + 1);
-  return launch_k(kernel, dim3(cluster, ntiles, (frames + 2 * np - 1) / (2 * np)), dim3(threads),
-                  smem, st, cluster, p, frames);
+  // eight compute warps whatever the plan's adj_warps: with four, eight pixels of
+  // four frames per thread take 165 registers
+  return launch_k(kernel, dim3(cluster, ntiles, (frames + 2 * np - 1) / (2 * np)),
+                  dim3(kAdjThreads), smem, st, cluster, p, frames);
 }
 
 // ---------------------------------------------------------------------------
@@ -1990,12 +1987,11 @@ cudaError_t configure_kernels(int smem_adj, int smem_fwd) {
   const int smem_frames = std::max(smem_adj, 88 * 1024);
   for (int dim = 2; dim <= 3; ++dim)
     for (int mode = ADJF_IMAGE; mode <= ADJF_BOTH; ++mode)
-      for (int warps = 4; warps <= 8; warps += 4)
-        for (int np = 1; np <= 2; ++np)
-          if ((e = cudaFuncSetAttribute(adjoint_frames_kernel(dim, mode, warps, np),
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        smem_frames)) != cudaSuccess)
-            return e;
+      for (int np = 1; np <= 2; ++np)
+        if ((e = cudaFuncSetAttribute(adjoint_frames_kernel(dim, mode, np),
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      smem_frames)) != cudaSuccess)
+          return e;
   const void* fwd[] = {
       (const void*)k_fwd_tile<2, false, 64>,  (const void*)k_fwd_tile<2, true, 64>,
       (const void*)k_fwd_tile<3, false, 64>,  (const void*)k_fwd_tile<3, true, 64>,

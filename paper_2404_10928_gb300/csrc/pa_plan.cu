@@ -65,6 +65,44 @@ static int num_sms(int dev) {
   return n > 0 ? n : 152;
 }
 
+// Work split of the gathers where the caller leaves it to the library.  Times:
+// pa_plan_time_gathers on a GB300 (152 SMs), 2D ring and 3D planar geometries.
+//
+// CTAs per tile in the adjoint.  2D: until two CTAs per SM exist (225 tiles, 400
+// sensors: 94 / 67 / 74 us with 1 / 2 / 4; 64 tiles, 256 sensors: 51 / 29 / 20 /
+// 18.5 with 1 / 2 / 4 / 8).  3D: at least two, which shorten the last wave (2048
+// tiles, 1024 sensors 1284 -> 1230 us; 675 tiles, 900 sensors 440 -> 419), and up
+// to 1000 CTAs (256 tiles, 400 sensors: 86 / 77 / 84 us with 2 / 4 / 8) while each
+// keeps a pipeline stage of 16 sensors (63 tiles, 64 sensors: 12.3 / 14.5 us with
+// 4 / 8).
+int default_cluster(int dim, int64_t ntiles, int S, int sms) {
+  int C = 1;
+  if (dim == 2) {
+    while (C < 8 && ntiles * C < 2LL * sms && 2 * C <= S) C *= 2;
+  } else {
+    while (C < 8 && (C == 1 || ntiles * C * 152 < 1000LL * sms) && S >= 32 * C) C *= 2;
+  }
+  return C;
+}
+
+// Compute warps of an adjoint CTA: four (eight pixels per thread) where a cluster
+// gives each CTA few sensors (2D: 64 tiles, 256 sensors 20.5 -> 18.5 us, 144 tiles,
+// 200 sensors 28.3 -> 26.6); eight otherwise (the same within 1% at two CTAs per
+// tile; 128^3 1260 against 1230 us).
+int default_adj_warps(int dim, int cluster) { return dim == 2 && cluster >= 4 ? 4 : 8; }
+
+// Sensors per forward work item: about 800 items where there is little work
+// (64^2, 64 sensors: 13.3 us with 8 sensors per item, 20.5 with 32; 301 x 187, 173
+// sensors: 24.6 with 12, 29.4 with 32), 24 until that gives about 4500 (384^2, 200
+// sensors: 45.1 with 24, 47.7 with 32; 64^3, 400 sensors: 126 with 24, 157 with
+// 128), then up to 128 (128^3, 1024 sensors: 2061 with 128, 2139 with 32).
+static int default_fwd_sensors(int64_t ntiles, int S, int sms) {
+  const int64_t units = ntiles * S * 152 / std::max(sms, 1);  // as on 152 SMs
+  const int64_t spc = units <= 24 * 4500 ? std::min<int64_t>(24, (units + 799) / 800)
+                                         : std::min<int64_t>(128, units / 4500);
+  return (int)std::max<int64_t>(8, (spc + 3) / 4 * 4);
+}
+
 // Builds the per-(tile, sensor) reference table for the plan's current c.
 static pa_status build_table(pa_plan* p) {
   const double kappa = p->fs / p->c;
@@ -332,13 +370,15 @@ pa_status pa_plan_create(pa_plan** out, const double* sensors_xyz, int n_sensors
   p->Kp = (p->K + 2 * p->pad + 1) / 2 * 2;
   {
     const int sms = num_sms(p->device);
-    int C = 1;
-    while (C < 8 && (int64_t)p->ntiles * C < 2LL * sms && 2 * C <= p->S) C *= 2;
-    p->cluster = C;
+    p->cluster = default_cluster(p->dim, p->ntiles, p->S, sms);
     if (opts && opts->adj_cluster > 0) p->cluster = std::min(opts->adj_cluster, p->S);
+    p->adj_warps = opts && opts->adj_warps > 0 ? opts->adj_warps
+                                               : default_adj_warps(p->dim, p->cluster);
+    p->fwd_spc = default_fwd_sensors(p->ntiles, p->S, sms);
+    if (forward_smem_bytes(p->dim, p->L, p->fwd_spc) > 200 * 1024)
+      p->fwd_spc = std::min(p->fwd_spc, kFwdSPC);
     if (opts && opts->fwd_sensors_per_cta > 0) p->fwd_spc = opts->fwd_sensors_per_cta;
     if (opts && opts->fwd_threads > 0) p->fwd_threads = opts->fwd_threads;
-    if (opts && opts->adj_warps > 0) p->adj_warps = opts->adj_warps;
     // the 4-sample combine reads 16-byte window slices per lane, and its warps span
     // 128 samples; once more than 16 windows cover a sample on average, lanes of a
     // warp mostly read different windows and one sample per lane (coalesced) wins

@@ -141,8 +141,7 @@ extern "C" pa_status pa_adjoint_static(const double* sensors_xyz, int n_sensors,
   PA_CUDA(cudaGetDevice(&dev));
   int sms = 152;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 152;
-  int C = 1;
-  while (C < 8 && ntiles * C < 2LL * sms && 2 * C <= n_sensors) C *= 2;
+  int C = default_cluster(dim, ntiles, n_sensors, sms);
   if (opts && opts->adj_cluster > 0) C = std::min(opts->adj_cluster, n_sensors);
 
   // scratch layout: flag | sensors | reference table | tap ranges | packed traces
@@ -203,7 +202,7 @@ extern "C" pa_status pa_adjoint_static(const double* sensors_xyz, int n_sensors,
   a.red = Reduce{};
   a.err = d_err;
   a.sensors_per_rank = (n_sensors + C - 1) / C;
-  a.warps = (opts && opts->adj_warps > 0) ? opts->adj_warps : kAdjWarps;
+  a.warps = (opts && opts->adj_warps > 0) ? opts->adj_warps : default_adj_warps(dim, C);
   PA_CUDA(launch_adjoint(dim, a, C, (int)ntiles, st));
   return PA_OK;
 }
