@@ -104,6 +104,13 @@ pa_status fwd_frames(pa_plan* p, int n, const float* x, float* out, int mode, co
   f.fs_trace = n_trace(p);
   f.fs_part = (int64_t)p->S * p->ntiles * p->L;
   f.fs_red = p->n_partials;
+  // the frames' items count like more sensors (8 frames of 256^2, 128 sensors: 68
+  // us with 24 or 32 sensors per item, 73 with one frame's 12), within the shared
+  // memory that the plan's kernels were set up for
+  f.spc = p->fwd_spc_frames > 0
+              ? p->fwd_spc_frames
+              : std::min(std::max(p->fwd_spc, kFwdSPC),
+                         default_fwd_sensors((int64_t)n * p->ntiles * p->S, 152));
   if (mode != FWD_STORE) f.red = stored_f(p->d_parts_f);
   PA_CUDA(launch_forward(p->dim, f, st, n));
   return PA_OK;

@@ -315,7 +315,8 @@ __host__ __device__ inline int combine_kblocks(int K, int threads, int spt) {
   return (K + spt * threads - 1) / (spt * threads);
 }
 pa_status validate_grid(const pa_grid* g);
-// the adjoint's work split where the caller leaves it open (pa_plan.cu)
+// the gathers' work split where the caller leaves it open (pa_plan.cu)
+int default_fwd_sensors(int64_t units, int sms);
 int default_cluster(int dim, int64_t ntiles, int S, int sms);
 int default_adj_warps(int dim, int cluster);
 
@@ -394,6 +395,7 @@ struct pa_plan {
   int fwd_threads = pa::kFwdThreadsDefault;  // threads per forward tile work item (64, 128, 256)
   int adj_warps = pa::kAdjWarps;             // compute warps per adjoint CTA (4 or 8)
   int comb_spt = 4; // samples per combine thread (1 when many windows cover a sample)
+  int fwd_spc_frames = 0;  // fwd_spc of a launch over several frames (0 = from its work)
 
   // device memory owned by the plan
   double* d_sensors = nullptr;

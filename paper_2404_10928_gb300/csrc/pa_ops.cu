@@ -1876,37 +1876,61 @@ __device__ __forceinline__ void combine_block(const FwdParams& P, int s, int kbl
     float v[SPT];
 #pragma unroll
     for (int j = 0; j < SPT; ++j) v[j] = 0.0f;
-    auto add = [&](int2 a) {
-      const float* src = ps + (int64_t)a.x * P.L + (k - a.y);
+    auto ok = [&](int2 a) {
 #ifdef PA_CHECKED
       if (k - a.y < 0 || k - a.y > P.L - SPT || a.x < 0 || a.x >= P.ntiles) {
         atomicOr(P.err, ERR_INDEX);
-        return;
+        return false;
       }
+#else
+      (void)a;
 #endif
-      if (SPT == 4) {
-        const float4 w = __ldcg(reinterpret_cast<const float4*>(src));
-        v[0] += w.x;
-        v[SPT > 1 ? 1 : 0] += w.y;
-        v[SPT > 2 ? 2 : 0] += w.z;
-        v[SPT > 3 ? 3 : 0] += w.w;
-      } else {
-        v[0] += __ldcg(src);
-      }
+      return true;
     };
-    // UNR independent loads in flight, summed in order: 4 where few windows
-    // cover a sample (SPT = 4), 16 where many do (SPT = 1: ~224 at 128^3, where
-    // 16 against 4 took the 30-CGLS reconstruction from 102.5 to 101.3 ms)
-    constexpr int UNR = SPT == 1 ? 16 : 4;
-    int i = i0;
-    for (; i + UNR <= i1; i += UNR) {
-      int2 e[UNR];
+    if (SPT == 4) {
+      // few windows per sample: rounds of eight, the last one as wide, with absent
+      // windows adding +0 (which does not change a sum that started at +0); with
+      // rounds of four and the rest one by one, each two dependent loads, the rest
+      // had been the longest part (256^2 ring 9.4 -> 7.6 us)
+      constexpr int kBatch = 8;
+      for (int i = i0; i < i1; i += kBatch) {
+        int2 e[kBatch];
+        float4 w[kBatch];
 #pragma unroll
-      for (int j = 0; j < UNR; ++j) e[j] = srt[i + j];
+        for (int j = 0; j < kBatch; ++j) e[j] = i + j < i1 ? srt[i + j] : make_int2(-1, 0);
 #pragma unroll
-      for (int j = 0; j < UNR; ++j) add(e[j]);
+        for (int j = 0; j < kBatch; ++j) {
+          w[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          if (e[j].x >= 0 && ok(e[j]))
+            w[j] = __ldcg(reinterpret_cast<const float4*>(ps + (int64_t)e[j].x * P.L + (k - e[j].y)));
+        }
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+          v[0] += w[j].x;
+          v[SPT > 1 ? 1 : 0] += w[j].y;
+          v[SPT > 2 ? 2 : 0] += w[j].z;
+          v[SPT > 3 ? 3 : 0] += w[j].w;
+        }
+      }
+    } else {
+      // many (~224 at 128^3): 16 loads in flight, summed in order (16 against 4 took
+      // the 30-CGLS reconstruction from 102.5 to 101.3 ms; rounds padded to 16, or a
+      // warp walking the windows of all its samples together, are 9% and 3-14%
+      // slower: issue)
+      constexpr int UNR = 16;
+      auto add = [&](int2 a) {
+        if (ok(a)) v[0] += __ldcg(ps + (int64_t)a.x * P.L + (k - a.y));
+      };
+      int i = i0;
+      for (; i + UNR <= i1; i += UNR) {
+        int2 e[UNR];
+#pragma unroll
+        for (int j = 0; j < UNR; ++j) e[j] = srt[i + j];
+#pragma unroll
+        for (int j = 0; j < UNR; ++j) add(e[j]);
+      }
+      for (; i < i1; ++i) add(srt[i]);
     }
-    for (; i < i1; ++i) add(srt[i]);
     const int64_t o = frame * P.fs_trace + (int64_t)s * P.K + k;
     const int n = min(SPT, P.K - k);
 #pragma unroll

@@ -96,8 +96,9 @@ int default_adj_warps(int dim, int cluster) { return dim == 2 && cluster >= 4 ? 
 // sensors: 24.6 with 12, 29.4 with 32), 24 until that gives about 4500 (384^2, 200
 // sensors: 45.1 with 24, 47.7 with 32; 64^3, 400 sensors: 126 with 24, 157 with
 // 128), then up to 128 (128^3, 1024 sensors: 2061 with 128, 2139 with 32).
-static int default_fwd_sensors(int64_t ntiles, int S, int sms) {
-  const int64_t units = ntiles * S * 152 / std::max(sms, 1);  // as on 152 SMs
+// units: (tile, sensor) pairs of the launch.
+int default_fwd_sensors(int64_t units, int sms) {
+  units = units * 152 / std::max(sms, 1);  // as on 152 SMs
   const int64_t spc = units <= 24 * 4500 ? std::min<int64_t>(24, (units + 799) / 800)
                                          : std::min<int64_t>(128, units / 4500);
   return (int)std::max<int64_t>(8, (spc + 3) / 4 * 4);
@@ -374,10 +375,11 @@ pa_status pa_plan_create(pa_plan** out, const double* sensors_xyz, int n_sensors
     if (opts && opts->adj_cluster > 0) p->cluster = std::min(opts->adj_cluster, p->S);
     p->adj_warps = opts && opts->adj_warps > 0 ? opts->adj_warps
                                                : default_adj_warps(p->dim, p->cluster);
-    p->fwd_spc = default_fwd_sensors(p->ntiles, p->S, sms);
+    p->fwd_spc = default_fwd_sensors((int64_t)p->ntiles * p->S, sms);
     if (forward_smem_bytes(p->dim, p->L, p->fwd_spc) > 200 * 1024)
       p->fwd_spc = std::min(p->fwd_spc, kFwdSPC);
-    if (opts && opts->fwd_sensors_per_cta > 0) p->fwd_spc = opts->fwd_sensors_per_cta;
+    if (opts && opts->fwd_sensors_per_cta > 0)
+      p->fwd_spc = p->fwd_spc_frames = opts->fwd_sensors_per_cta;
     if (opts && opts->fwd_threads > 0) p->fwd_threads = opts->fwd_threads;
     // the 4-sample combine reads 16-byte window slices per lane, and its warps span
     // 128 samples; once more than 16 windows cover a sample on average, lanes of a
@@ -385,7 +387,9 @@ pa_status pa_plan_create(pa_plan** out, const double* sensors_xyz, int n_sensors
     p->comb_spt = (int64_t)p->ntiles * p->L <= 16 * (int64_t)p->K ? 4 : 1;
   }
   const size_t smem_adj = (size_t)adjoint_smem_bytes(p->L);
-  const size_t smem_fwd = (size_t)forward_smem_bytes(p->dim, p->L, p->fwd_spc);
+  // launches over several frames take up to kFwdSPC sensors per item by themselves
+  const size_t smem_fwd = (size_t)forward_smem_bytes(
+      p->dim, p->L, p->fwd_spc_frames > 0 ? p->fwd_spc : std::max(p->fwd_spc, kFwdSPC));
   if (smem_adj > 200 * 1024 || smem_fwd > 200 * 1024) {
     set_error("geometry needs too much shared memory (window %d samples, %d tiles)", p->L,
               p->ntiles);
