@@ -11,6 +11,7 @@ namespace pa {
 FwdParams forward_params(const pa_plan* p, const float* x, float* out, int mode, const void* y);
 AdjParams adjoint_params(const pa_plan* p, float* out, int mode, const double* omega, int nonneg);
 Reduce make_reduce(const pa_plan* p, int op, double* out_sum, const double* other, double* out2);
+void pack_into(const pa_plan* p, FwdParams& f);
 }  // namespace pa
 
 using namespace pa;
@@ -102,7 +103,7 @@ pa_status pa_batch_create(pa_batch** out, pa_plan* const* plans, int n_frames) {
   for (int f = 0; f < n_frames; ++f) {
     const pa_plan* p = plans[f];
     const int chunks = (p->S + kBatchFwdSensors - 1) / kBatchFwdSensors;
-    const int nk = combine_kblocks(p->K, kBatchThreads, 4);
+    const int nk = combine_kblocks(p->K, kBatchThreads, 4, true);
     pre[f + 1] = pre[f] + p->ntiles * chunks;
     pre[(n_frames + 1) + f + 1] = pre[(n_frames + 1) + f] + p->S * nk;
     pre[2 * (n_frames + 1) + f + 1] = pre[2 * (n_frames + 1) + f] + p->ntiles;
@@ -193,7 +194,7 @@ CglsLayout cgls_layout(const pa_plan* p, int n_iter) {
   CglsLayout L{};
   const size_t SK = (size_t)p->S * p->K * sizeof(float);
   const size_t N = (size_t)p->grid.nx * p->grid.ny * p->grid.nz * sizeof(float);
-  const int nk = combine_kblocks(p->K, kBatchThreads, 4);
+  const int nk = combine_kblocks(p->K, kBatchThreads, 4, true);
   L.n_xr = p->S * combine_kblocks(p->K, kBatchXrThreads, 4);
   L.h_stride = std::max(p->S * nk, L.n_xr);
   size_t o = 0;
@@ -335,11 +336,12 @@ pa_status pa_batch_landweber(pa_batch* b, int n_iter, const void* const* y_dev,
     BatchFrame& F = frames[f];
     std::memset(&F, 0, sizeof(F));
     F.f = forward_params(p, x_dev[f], b->d_r[f], FWD_RESID, y_dev[f]);
+    pack_into(p, F.f);
     F.f.red = make_reduce(p, OP_SUM, nullptr, nullptr, nullptr);
     F.a = adjoint_params(p, x_dev[f], ADJ_LANDWEBER, b->d_omega + f, nonneg);
     F.f.spc = kBatchFwdSensors;  // the batch's own forward items (see kBatchFwdSensors)
     F.fwd_chunks = (p->S + kBatchFwdSensors - 1) / kBatchFwdSensors;
-    F.n_kblk = combine_kblocks(p->K, kBatchThreads, 4);
+    F.n_kblk = combine_kblocks(p->K, kBatchThreads, 4, true);
     F.hist = b->d_hist + (size_t)f * (n_iter + 1);
   }
   return run_batch(b, PA_LANDWEBER, frames, omega, n_iter, residual_history_host, st,
@@ -394,10 +396,11 @@ pa_status pa_batch_reconstruct(pa_batch* b, pa_method method, int n_iter,
     F.N = p->grid.nx * p->grid.ny * p->grid.nz;
     F.nonneg = nonneg;
     F.f = forward_params(p, x_dev[f], F.rbuf[0], FWD_RESID, y_dev[f]);
+    pack_into(p, F.f);
     F.a = adjoint_params(p, F.s, ADJ_NORM, nullptr, 0);
     F.f.spc = kBatchFwdSensors;  // the batch's own forward items (see kBatchFwdSensors)
     F.fwd_chunks = (p->S + kBatchFwdSensors - 1) / kBatchFwdSensors;
-    F.n_kblk = combine_kblocks(p->K, kBatchThreads, 4);
+    F.n_kblk = combine_kblocks(p->K, kBatchThreads, 4, true);
     F.hist = b->d_hist + (size_t)f * (n_iter + 1);
   }
   return run_batch(b, PA_CGLS, frames, nullptr, n_iter, residual_history_host, st,

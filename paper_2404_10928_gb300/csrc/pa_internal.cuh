@@ -161,11 +161,12 @@ struct AdjParams {
   int sensors_per_rank;
   int warps;              // compute warps of k_adjoint: 4 or 8 (0 = 8)
   // ADJ_FISTA (out = x_k, updated in place; omega = the step tau): with g =
-  // A^T r, r = y - A z, v = z + tau (2 g - tv_beta tvg), x_new = prox(v), and
-  // z = x_new + mu (x_new - x_k), both in place
-  float* z;
-  const float* tvg;       // gradient of TV_eps at z (ADJ_FISTA), or the TV term (ADJ_AXPY)
-  float l1, tv_beta, mu;
+  // A^T r, r = y - A z, v = z + tau (2 g - tv_beta grad TV_eps(z)), x_new = prox(v),
+  // and z_out = x_new + mu (x_new - x_k)
+  const float* z;
+  float* z_out;
+  const float* tvg;       // the TV term (ADJ_AXPY)
+  float l1, tv_beta, tv_eps2, mu;
   float coef, tvw;        // ADJ_AXPY weights of A^T p and of tvg
   const float* dc_x;      // launch_adjoint_frames: images weighting the slopes, or null
   int64_t fs_img;         // launch_adjoint_frames: stride between frames' images, N
@@ -189,6 +190,10 @@ struct FwdParams {
   const void* y;          // [S][K] measured traces (FWD_RESID), f32 or f16
   int y_f16;
   Reduce red;             // ||out||^2 (FWD_RESID / FWD_NORM)
+  // the result also (out may then be null) as the adjoint's packed traces, written
+  // by the combine: [S][Kp] (mid, slope), rows starting pad samples in
+  float2* packed;
+  int Kp, pad;
   // optional CGLS direction update fused into the gather: the image applied is
   // x = s + beta p_old (s_in != nullptr), written to p_new by sensor chunk 0
   const float* s_in;
@@ -308,11 +313,14 @@ cudaError_t launch_forward(int dim, const FwdParams& p, cudaStream_t st, int fra
 int adjoint_smem_bytes(int L);
 cudaError_t configure_kernels(int smem_adj, int smem_fwd);
 int forward_smem_bytes(int dim, int L, int spc);
-int forward_combine_blocks(int S, int K, int spt);
+int forward_combine_blocks(int S, int K, int spt, bool pack = false);
 // sample blocks per sensor of the combine (and of the CGLS r update) when each
 // thread forms spt consecutive samples
-__host__ __device__ inline int combine_kblocks(int K, int threads, int spt) {
-  return (K + spt * threads - 1) / (spt * threads);
+// (a combine that packs: 31 groups per warp, the last lane only evaluates the
+// next warp's first group)
+__host__ __device__ inline int combine_kblocks(int K, int threads, int spt, bool pack = false) {
+  const int per = spt * (pack ? threads / 32 * 31 : threads);
+  return (K + per - 1) / per;
 }
 pa_status validate_grid(const pa_grid* g);
 // the gathers' work split where the caller leaves it open (pa_plan.cu)

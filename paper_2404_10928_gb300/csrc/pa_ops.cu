@@ -924,9 +924,57 @@ __device__ __forceinline__ float* adj_accumulate(const AdjParams& P, const float
   return s_acc;
 }
 
-// NW compute warps (kTilePixels / (32 NW) pixels per thread) and one producer warp
-template <int DIM, bool DC, int NW>
-__global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint(const AdjParams P) {
+// Terms of the smoothed TV (see k_tv) of pixel (i, j, l): its forward differences
+// over m = sqrt(their squares + eps^2).
+template <int DIM>
+__device__ __forceinline__ void tv_terms(const float* x, int i, int j, int l, int nx,
+                                         int ny, int nz, float eps2, float& ax, float& ay,
+                                         float& az, float& m) {
+  const int64_t o = ((int64_t)l * ny + j) * nx + i;
+  const float c = x[o];
+  const float gx = (i + 1 < nx) ? x[o + 1] - c : 0.0f;
+  const float gy = (j + 1 < ny) ? x[o + nx] - c : 0.0f;
+  const float gz = (DIM == 3 && l + 1 < nz) ? x[o + (int64_t)nx * ny] - c : 0.0f;
+  m = sqrtf(fmaf(gx, gx, fmaf(gy, gy, fmaf(gz, gz, eps2))));
+  const float inv = 1.0f / m;
+  ax = gx * inv;
+  ay = gy * inv;
+  az = gz * inv;
+}
+
+// The TV gradient at pixel (i, j, l), and its own term m of the value.
+template <int DIM>
+__device__ __forceinline__ float tv_gradient(const float* x, int i, int j, int l, int nx, int ny,
+                                             int nz, float eps2, float& m) {
+  float ax, ay, az;
+  tv_terms<DIM>(x, i, j, l, nx, ny, nz, eps2, ax, ay, az, m);
+  float g = -(ax + ay + az);
+  float bx, by, bz, mm;
+  if (i > 0) {
+    tv_terms<DIM>(x, i - 1, j, l, nx, ny, nz, eps2, bx, by, bz, mm);
+    g += bx;
+  }
+  if (j > 0) {
+    tv_terms<DIM>(x, i, j - 1, l, nx, ny, nz, eps2, bx, by, bz, mm);
+    g += by;
+  }
+  if (DIM == 3 && l > 0) {
+    tv_terms<DIM>(x, i, j, l - 1, nx, ny, nz, eps2, bx, by, bz, mm);
+    g += bz;
+  }
+  return g;
+}
+
+// NW compute warps (kTilePixels / (32 NW) pixels per thread) and one producer warp.
+// FISTA has its own kernels: its epilogue evaluates the TV gradient at z, which
+// took a launch of its own per iteration (256^2 ring, 20 iterations: 960 -> 916 us; as a
+// parallel branch of the graph it had cost 40 us more than in line).  Four CTAs per
+// SM as the other kinds: the epilogue's registers must not cost the gather one.
+enum AdjKind : int { ADJK_IMAGE = 0, ADJK_DC = 1, ADJK_FISTA = 2 };
+template <int DIM, int KIND, int NW>
+__global__ void __launch_bounds__(32 * (NW + 1), KIND == ADJK_FISTA && NW == 8 ? 4 : 2)
+    k_adjoint(const AdjParams P) {
+  constexpr bool DC = KIND == ADJK_DC;
   constexpr int NT = 32 * (NW + 1);
   constexpr int TX = Tile<DIM>::X, TY = Tile<DIM>::Y, TZ = Tile<DIM>::Z;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -965,6 +1013,20 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint(const AdjParams P)
       const float gval = P.amp * v;
       if (DC) {
         part = df_add(part, df_prod(xin[i], v));
+      } else if (KIND == ADJK_FISTA) {
+        // gradient step on ||A z - y||^2 + beta TV(z) at z, proximal step of
+        // tau l1 ||.||_1 (and x >= 0), then the extrapolation
+        const float tau = (float)(*P.omega);
+        const float zi = P.z[i];
+        float tvg = zi, m;  // unused when tv_beta = 0
+        if (P.tv_beta != 0.0f)
+          tvg = tv_gradient<DIM>(P.z, gx, gy, gz, P.g.nx, P.g.ny, P.g.nz, P.tv_eps2, m);
+        const float v = fmaf(tau, fmaf(2.0f, gval, -P.tv_beta * tvg), zi);
+        const float thr = tau * P.l1;
+        const float xn = P.nonneg ? fmaxf(v - thr, 0.0f) : copysignf(fmaxf(fabsf(v) - thr, 0.0f), v);
+        const float xo = out[i];
+        out[i] = xn;
+        P.z_out[i] = fmaf(P.mu, xn - xo, xn);
       } else if (P.mode == ADJ_LANDWEBER) {
         float xv = fmaf((float)(*P.omega), gval, out[i]);
         if (P.nonneg) xv = fmaxf(xv, 0.0f);
@@ -974,17 +1036,6 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint(const AdjParams P)
         if (P.tvg) xv = fmaf(P.tvw, P.tvg[i], xv);
         if (P.nonneg) xv = fmaxf(xv, 0.0f);
         out[i] = xv;
-      } else if (P.mode == ADJ_FISTA) {
-        // gradient step on ||A z - y||^2 + beta TV(z) at z, proximal step of
-        // tau l1 ||.||_1 (and x >= 0), then the extrapolation
-        const float tau = (float)(*P.omega);
-        const float zi = P.z[i];
-        const float v = fmaf(tau, fmaf(2.0f, gval, -P.tv_beta * P.tvg[i]), zi);
-        const float thr = tau * P.l1;
-        const float xn = P.nonneg ? fmaxf(v - thr, 0.0f) : copysignf(fmaxf(fabsf(v) - thr, 0.0f), v);
-        const float xo = P.out[i];
-        P.out[i] = xn;
-        P.z[i] = fmaf(P.mu, xn - xo, xn);
       } else {
         out[i] = gval;
         part = df_add(part, df_sq(gval));
@@ -1011,18 +1062,23 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint(const AdjParams P)
   (void)TZ;
 }
 
+using AdjKernel = void (*)(const AdjParams);
+template <int D, int W>
+AdjKernel adjoint_kernel(int kind) {
+  return kind == ADJK_DC      ? k_adjoint<D, ADJK_DC, W>
+         : kind == ADJK_FISTA ? k_adjoint<D, ADJK_FISTA, W>
+                              : k_adjoint<D, ADJK_IMAGE, W>;
+}
+AdjKernel adjoint_kernel(int dim, int kind, int warps) {
+  return dim == 2 ? (warps == 4 ? adjoint_kernel<2, 4>(kind) : adjoint_kernel<2, kAdjWarps>(kind))
+                  : (warps == 4 ? adjoint_kernel<3, 4>(kind) : adjoint_kernel<3, kAdjWarps>(kind));
+}
+
 cudaError_t launch_adjoint(int dim, const AdjParams& p, int cluster, int ntiles, cudaStream_t st) {
-  const bool dc = p.mode == ADJ_DC;
-  if (p.warps == 4) {
-    auto kernel = dim == 2 ? (dc ? k_adjoint<2, true, 4> : k_adjoint<2, false, 4>)
-                           : (dc ? k_adjoint<3, true, 4> : k_adjoint<3, false, 4>);
-    return launch_k(kernel, dim3(cluster, ntiles), dim3(32 * 5), adjoint_smem_bytes(p.L),
-                    st, cluster, p);
-  }
-  auto kernel = dim == 2 ? (dc ? k_adjoint<2, true, kAdjWarps> : k_adjoint<2, false, kAdjWarps>)
-                         : (dc ? k_adjoint<3, true, kAdjWarps> : k_adjoint<3, false, kAdjWarps>);
-  return launch_k(kernel, dim3(cluster, ntiles), dim3(kAdjThreads), adjoint_smem_bytes(p.L),
-                  st, cluster, p);
+  const int kind = p.mode == ADJ_DC ? ADJK_DC : p.mode == ADJ_FISTA ? ADJK_FISTA : ADJK_IMAGE;
+  const int warps = p.warps == 4 ? 4 : kAdjWarps;
+  return launch_k(adjoint_kernel(dim, kind, warps), dim3(cluster, ntiles), dim3(32 * (warps + 1)),
+                  adjoint_smem_bytes(p.L), st, cluster, p);
 }
 
 // ---------------------------------------------------------------------------
@@ -1861,21 +1917,31 @@ __global__ void __launch_bounds__(NT) k_fwd_tile(const FwdParams P) {
 // the same windows (coalesced) — the better choice when many windows cover
 // each sample (large 3D grids).  nkblk = sample blocks per sensor (for the
 // in-kernel reduction's slot numbering).
-template <int MODE, int SPT>
+//   PACK: the result goes to the adjoint's packed (mid, slope) rows as well (or
+// only there), the pass of k_pack: entry k needs sample k + 1, so a warp's last
+// lane evaluates the first samples of the next warp and stores nothing (3% more
+// gathers against one launch and 12 bytes per sample of traffic: 20 FISTA
+// iterations of the 256^2 ring 1013 -> 960 us).
+template <int MODE, int SPT, bool PACK = false>
 __device__ __forceinline__ void combine_block(const FwdParams& P, int s, int kblk, int nkblk,
                                               int frame = 0) {
   static_assert(SPT == 1 || SPT == 4, "1 or 4 samples per thread");
   __shared__ DF s_red[32];
-  const int k = SPT * (kblk * blockDim.x + threadIdx.x);
+  const int lane = threadIdx.x & 31;
+  const int k = PACK ? SPT * ((kblk * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 31 + lane)
+                     : SPT * (kblk * blockDim.x + threadIdx.x);
+  const bool halo = PACK && lane == 31;
   DF part = df_zero();
+  float v[SPT];
+#pragma unroll
+  for (int j = 0; j < SPT; ++j) v[j] = 0.0f;
+  const int n = min(SPT, P.K - k);  // samples of this thread (none past the row)
+  const int64_t o = frame * P.fs_trace + (int64_t)s * P.K + k;
   if (k < P.K) {
     const int* up = P.upper + (int64_t)s * (P.K + P.L);
     const int i0 = up[k], i1 = up[k + P.L];  // windows starting in (k - L, k]
     const int2* srt = P.sorted + (int64_t)s * P.ntiles;
     const float* ps = P.part + frame * P.fs_part + (int64_t)s * P.ntiles * P.L;
-    float v[SPT];
-#pragma unroll
-    for (int j = 0; j < SPT; ++j) v[j] = 0.0f;
     auto ok = [&](int2 a) {
 #ifdef PA_CHECKED
       if (k - a.y < 0 || k - a.y > P.L - SPT || a.x < 0 || a.x >= P.ntiles) {
@@ -1931,8 +1997,6 @@ __device__ __forceinline__ void combine_block(const FwdParams& P, int s, int kbl
       }
       for (; i < i1; ++i) add(srt[i]);
     }
-    const int64_t o = frame * P.fs_trace + (int64_t)s * P.K + k;
-    const int n = min(SPT, P.K - k);
 #pragma unroll
     for (int j = 0; j < SPT; ++j) {
       v[j] *= P.amp;
@@ -1942,17 +2006,42 @@ __device__ __forceinline__ void combine_block(const FwdParams& P, int s, int kbl
         v[j] = y - v[j];
       }
     }
-    if (SPT == 4 && n == 4 && (P.K & 3) == 0) {
-      *reinterpret_cast<float4*>(P.out + o) =
-          make_float4(v[0], v[SPT > 1 ? 1 : 0], v[SPT > 2 ? 2 : 0], v[SPT > 3 ? 3 : 0]);
-    } else {
+    if (!halo && (!PACK || P.out)) {
+      if (SPT == 4 && n == 4 && (P.K & 3) == 0) {
+        *reinterpret_cast<float4*>(P.out + o) =
+            make_float4(v[0], v[SPT > 1 ? 1 : 0], v[SPT > 2 ? 2 : 0], v[SPT > 3 ? 3 : 0]);
+      } else {
 #pragma unroll
-      for (int j = 0; j < SPT; ++j)
-        if (j < n) P.out[o + j] = v[j];
+        for (int j = 0; j < SPT; ++j)
+          if (j < n) P.out[o + j] = v[j];
+      }
     }
 #pragma unroll
     for (int j = 0; j < SPT; ++j)
-      if (j < n) part = df_add(part, df_sq(v[j]));
+      if (j < n && !halo) part = df_add(part, df_sq(v[j]));
+  }
+  if (PACK) {
+    float r[SPT + 1];
+#pragma unroll
+    for (int j = 0; j < SPT; ++j) r[j] = j < n ? v[j] : 0.0f;  // r_K = 0
+    r[SPT] = __shfl_down_sync(0xffffffffu, r[0], 1);
+    if (!halo && n > 0) {
+      float2* row = P.packed + (int64_t)s * P.Kp + P.pad + k;
+      if (k == 0) row[-1] = make_float2(0.5f * r[0], r[0]);
+      if (SPT == 4 && n == 4) {
+        // pad, Kp and k are even: two 16-byte stores of two (mid, slope) each
+        constexpr int q1 = SPT > 1 ? 1 : 0, q2 = SPT > 2 ? 2 : 0, q3 = SPT > 3 ? 3 : 0;
+        float4* dst = reinterpret_cast<float4*>(row);
+        dst[0] = make_float4(0.5f * (r[0] + r[q1]), r[q1] - r[0], 0.5f * (r[q1] + r[q2]),
+                             r[q2] - r[q1]);
+        dst[1] = make_float4(0.5f * (r[q2] + r[q3]), r[q3] - r[q2], 0.5f * (r[q3] + r[SPT]),
+                             r[SPT] - r[q3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < SPT; ++j)
+          if (j < n) row[j] = make_float2(0.5f * (r[j] + r[j + 1]), r[j + 1] - r[j]);
+      }
+    }
   }
   if (MODE != FWD_STORE) {
     const DF t = block_sum(part, s_red, blockDim.x >> 5);
@@ -1960,12 +2049,14 @@ __device__ __forceinline__ void combine_block(const FwdParams& P, int s, int kbl
   }
 }
 
-template <int MODE, int SPT>
+template <int MODE, int SPT, bool PACK>
 __global__ void __launch_bounds__(kCombThreads) k_fwd_combine(const FwdParams P) {
-  combine_block<MODE, SPT>(P, blockIdx.y, blockIdx.x, gridDim.x, blockIdx.z);
+  combine_block<MODE, SPT, PACK>(P, blockIdx.y, blockIdx.x, gridDim.x, blockIdx.z);
 }
 
-int forward_combine_blocks(int S, int K, int spt) { return S * combine_kblocks(K, kCombThreads, spt); }
+int forward_combine_blocks(int S, int K, int spt, bool pack) {
+  return S * combine_kblocks(K, kCombThreads, spt, pack);
+}
 
 cudaError_t launch_forward(int dim, const FwdParams& p, cudaStream_t st, int frames) {
   const int smem = forward_smem_bytes(dim, p.L, p.spc);
@@ -1982,14 +2073,19 @@ cudaError_t launch_forward(int dim, const FwdParams& p, cudaStream_t st, int fra
                                  : pick(std::integral_constant<int, 128>());
   const cudaError_t e = launch_k(tile_kernel, grid1, dim3(nt), smem, st, 0, p);
   if (e != cudaSuccess) return e;
-  const dim3 grid2(combine_kblocks(p.K, kCombThreads, p.comb_spt), p.S, frames);
-  auto combine = p.comb_spt == 4
-                     ? (p.mode == FWD_RESID ? k_fwd_combine<FWD_RESID, 4>
-                        : p.mode == FWD_NORM ? k_fwd_combine<FWD_NORM, 4>
-                                             : k_fwd_combine<FWD_STORE, 4>)
-                     : (p.mode == FWD_RESID ? k_fwd_combine<FWD_RESID, 1>
-                        : p.mode == FWD_NORM ? k_fwd_combine<FWD_NORM, 1>
-                                             : k_fwd_combine<FWD_STORE, 1>);
+  const bool pack = p.packed != nullptr;
+  const dim3 grid2(combine_kblocks(p.K, kCombThreads, p.comb_spt, pack), p.S, frames);
+  auto pick_combine = [&](auto spt) {
+    constexpr int SPT = decltype(spt)::value;
+    if (pack)
+      return p.mode == FWD_RESID ? k_fwd_combine<FWD_RESID, SPT, true>
+                                 : k_fwd_combine<FWD_STORE, SPT, true>;
+    return p.mode == FWD_RESID  ? k_fwd_combine<FWD_RESID, SPT, false>
+           : p.mode == FWD_NORM ? k_fwd_combine<FWD_NORM, SPT, false>
+                                : k_fwd_combine<FWD_STORE, SPT, false>;
+  };
+  auto combine = p.comb_spt == 4 ? pick_combine(std::integral_constant<int, 4>())
+                                 : pick_combine(std::integral_constant<int, 1>());
   return launch_k(combine, grid2, dim3(kCombThreads), 0, st, 0, p);
 }
 
@@ -1997,15 +2093,13 @@ cudaError_t launch_forward(int dim, const FwdParams& p, cudaStream_t st, int fra
 // plan is created, outside any stream capture).
 cudaError_t configure_kernels(int smem_adj, int smem_fwd) {
   cudaError_t e;
-  const void* adj[] = {
-      (const void*)k_adjoint<2, false, 4>, (const void*)k_adjoint<2, true, 4>,
-      (const void*)k_adjoint<3, false, 4>, (const void*)k_adjoint<3, true, 4>,
-      (const void*)k_adjoint<2, false, kAdjWarps>, (const void*)k_adjoint<2, true, kAdjWarps>,
-      (const void*)k_adjoint<3, false, kAdjWarps>, (const void*)k_adjoint<3, true, kAdjWarps>};
-  for (const void* k : adj)
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_adj)) !=
-        cudaSuccess)
-      return e;
+  for (int dim = 2; dim <= 3; ++dim)
+    for (int kind = ADJK_IMAGE; kind <= ADJK_FISTA; ++kind)
+      for (int warps = 4; warps <= 8; warps += 4)
+        if ((e = cudaFuncSetAttribute(adjoint_kernel(dim, kind, warps),
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem_adj)) !=
+            cudaSuccess)
+          return e;
   // the frames' gathers take at most the single-frame gather's windows, or 80 KB of
   // stages (adjf_stages)
   const int smem_frames = std::max(smem_adj, 88 * 1024);
@@ -2376,22 +2470,6 @@ cudaError_t launch_norm(const float* v, int64_t n, const Reduce& red, int nblk, 
 // every frame's (eight 256^2 frames: 8 launches of 7.7 us -> one of 13 us).
 // ---------------------------------------------------------------------------
 template <int DIM>
-__device__ __forceinline__ void tv_terms(const float* x, int i, int j, int l, int nx,
-                                         int ny, int nz, float eps2, float& ax, float& ay,
-                                         float& az, float& m) {
-  const int64_t o = ((int64_t)l * ny + j) * nx + i;
-  const float c = x[o];
-  const float gx = (i + 1 < nx) ? x[o + 1] - c : 0.0f;
-  const float gy = (j + 1 < ny) ? x[o + nx] - c : 0.0f;
-  const float gz = (DIM == 3 && l + 1 < nz) ? x[o + (int64_t)nx * ny] - c : 0.0f;
-  m = sqrtf(fmaf(gx, gx, fmaf(gy, gy, fmaf(gz, gz, eps2))));
-  const float inv = 1.0f / m;
-  ax = gx * inv;
-  ay = gy * inv;
-  az = gz * inv;
-}
-
-template <int DIM>
 __global__ void __launch_bounds__(kVecThreads) k_tv(const float* images, int nx, int ny,
                                                     int nz, float eps, float* grads,
                                                     const Reduce red) {
@@ -2404,24 +2482,9 @@ __global__ void __launch_bounds__(kVecThreads) k_tv(const float* images, int nx,
   for (int64_t o = blockIdx.x * (int64_t)kVecThreads + threadIdx.x; o < n;
        o += (int64_t)gridDim.x * kVecThreads) {
     const int i = (int)(o % nx), j = (int)((o / nx) % ny), l = (int)(o / ((int64_t)nx * ny));
-    float ax, ay, az, m;
-    tv_terms<DIM>(x, i, j, l, nx, ny, nz, eps2, ax, ay, az, m);
+    float m;
+    grad[o] = tv_gradient<DIM>(x, i, j, l, nx, ny, nz, eps2, m);
     part = df_add(part, df_of(m));
-    float g = -(ax + ay + az);
-    float bx, by, bz, mm;
-    if (i > 0) {
-      tv_terms<DIM>(x, i - 1, j, l, nx, ny, nz, eps2, bx, by, bz, mm);
-      g += bx;
-    }
-    if (j > 0) {
-      tv_terms<DIM>(x, i, j - 1, l, nx, ny, nz, eps2, bx, by, bz, mm);
-      g += by;
-    }
-    if (DIM == 3 && l > 0) {
-      tv_terms<DIM>(x, i, j, l - 1, nx, ny, nz, eps2, bx, by, bz, mm);
-      g += bz;
-    }
-    grad[o] = g;
   }
   const DF t = block_sum<kVecThreads / 32>(part, s_red);
   if (gridDim.y == 1) {
@@ -2477,8 +2540,8 @@ cudaError_t launch_tv_frames(int dim, const float* x, int nx, int ny, int nz, fl
 // Batched projected Landweber over frames of uneven size, in one persistent
 // cooperative launch (co-residency of all CTAs is guaranteed by the launch).
 // Per iteration: every frame's forward tile items, then its combine items
-// (r = y - A x and ||r||^2), then the packing of r, then its adjoint items with
-// the Landweber update.  Items come from one global queue per phase, so CTAs
+// (r = y - A x, packed, and ||r||^2), then its adjoint items with the Landweber
+// update.  Items come from one global queue per phase, so CTAs
 // balance the ragged work among themselves; every item's arithmetic is the
 // same as in the single-frame kernels.  Phases are separated by a grid barrier
 // whose wait is bounded: if it gives up, an error flag is set and the CTA goes
@@ -2580,26 +2643,10 @@ __global__ void __launch_bounds__(kBatchThreads, 4) k_batch_landweber(
       FwdParams P = frames[f].f;
       P.red.out_sum = frames[f].hist + it;
       const int nk = frames[f].n_kblk;
-      combine_block<FWD_RESID, 4>(P, li / nk, li % nk, nk);
+      combine_block<FWD_RESID, 4, true>(P, li / nk, li % nk, nk);
     }
     grid_barrier(state, nb, err, state + 3, wait_ns);
     if (it == n_iter) break;
-    for (int f = 0; f < nf; ++f) {  // pack r of every frame (grid-stride)
-      const FwdParams& F = frames[f].f;
-      const AdjParams& A = frames[f].a;
-      const int64_t row = F.K + 1, total = (int64_t)F.S * row;
-      for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-           idx += (int64_t)gridDim.x * blockDim.x) {
-        const int s = (int)(idx / row);
-        const int k = (int)(idx % row) - 1;
-        const float* rs = F.out + (int64_t)s * F.K;
-        const float a = (k >= 0) ? rs[k] : 0.0f;
-        const float b = (k + 1 < F.K) ? rs[k + 1] : 0.0f;
-        const_cast<float2*>(A.packed)[(int64_t)s * A.Kp + A.pad + k] =
-            make_float2(0.5f * (a + b), b - a);
-      }
-    }
-    grid_barrier(state, nb, err, nullptr, wait_ns);
     for (int gi = grab_item(state + 4); gi < pa[nf]; gi = grab_item(state + 4)) {
       const int f = frame_of(pa, nf, gi);
       adj_landweber_block<DIM>(frames[f].a, gi - pa[f], smem);
@@ -2675,25 +2722,9 @@ __global__ void __launch_bounds__(kBatchThreads, 4) k_batch_cgls(
     P.out = frames[f].rbuf[0];
     P.red = stored_parts(frames[f].h_parts);
     const int nk = frames[f].n_kblk;
-    combine_block<FWD_RESID, 4>(P, li / nk, li % nk, nk);
+    combine_block<FWD_RESID, 4, true>(P, li / nk, li % nk, nk);
   }
   grid_barrier(state, nb, err, state + 3, wait_ns);
-  for (int f = 0; f < nf; ++f) {  // pack r_0 of every frame (grid-stride)
-    const FwdParams& F = frames[f].f;
-    const AdjParams& A = frames[f].a;
-    const float* rs0 = frames[f].rbuf[0];
-    const int64_t row = F.K + 1, total = (int64_t)F.S * row;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-      const int s = (int)(idx / row);
-      const int k = (int)(idx % row) - 1;
-      const float* rs = rs0 + (int64_t)s * F.K;
-      const float a = (k >= 0) ? rs[k] : 0.0f;
-      const float b = (k + 1 < F.K) ? rs[k + 1] : 0.0f;
-      const_cast<float2*>(A.packed)[(int64_t)s * A.Kp + A.pad + k] = make_float2(0.5f * (a + b), b - a);
-    }
-  }
-  grid_barrier(state, nb, err, nullptr, wait_ns);
   for (int gi = grab_item(state + 4); gi < pa[nf]; gi = grab_item(state + 4)) {
     const int f = frame_of(pa, nf, gi);
     adj_norm_block<DIM>(frames[f].a, gi - pa[f], frames[f].pbuf[0], frames[f].s_parts, smem);

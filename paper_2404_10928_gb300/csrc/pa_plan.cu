@@ -421,7 +421,7 @@ pa_status pa_plan_create(pa_plan** out, const double* sensors_xyz, int n_sensors
   const size_t n_pix = (size_t)grid->nx * grid->ny * grid->nz;
   const size_t n_tr = (size_t)p->S * p->K;
   p->n_partials = (int)std::max<int64_t>(
-      {(int64_t)p->ntiles * p->cluster, (int64_t)forward_combine_blocks(p->S, p->K, 1),
+      {(int64_t)p->ntiles * p->cluster, (int64_t)forward_combine_blocks(p->S, p->K, 1, true),
        (int64_t)cgls_r_blocks(p->S, p->K), 152 * 8, 1});
   if (cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
@@ -576,6 +576,13 @@ FwdParams forward_params(const pa_plan* p, const float* x, float* out, int mode,
   f.red = Reduce{};
   f.err = p->d_err;
   return f;
+}
+
+// the combine writes its result into the plan's packed traces too
+void pack_into(const pa_plan* p, FwdParams& f) {
+  f.packed = p->d_packed;
+  f.Kp = p->Kp;
+  f.pad = p->pad;
 }
 
 AdjParams adjoint_params(const pa_plan* p, float* out, int mode, const double* omega, int nonneg) {

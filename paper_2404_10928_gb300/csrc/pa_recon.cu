@@ -13,6 +13,7 @@ namespace pa {
 FwdParams forward_params(const pa_plan* p, const float* x, float* out, int mode, const void* y);
 AdjParams adjoint_params(const pa_plan* p, float* out, int mode, const double* omega, int nonneg);
 Reduce make_reduce(const pa_plan* p, int op, double* out_sum, const double* other, double* out2);
+void pack_into(const pa_plan* p, FwdParams& f);
 
 namespace {
 
@@ -150,10 +151,12 @@ Reduce stored(float2* parts) {
   return r;
 }
 
+// pack: the result also as the plan's packed traces (out may then be NULL).
 pa_status fwd(pa_plan* p, const float* x, float* out, int mode, const void* y, const Reduce& red,
-              Timing& t, cudaStream_t st, const DirUpdate& du = DirUpdate()) {
+              Timing& t, cudaStream_t st, const DirUpdate& du = DirUpdate(), bool pack = false) {
   PA_TRY(mark(t, true, st));
   FwdParams f = forward_params(p, du.s ? nullptr : x, out, mode, y);
+  if (pack) pack_into(p, f);
   f.red = red;
   f.s_in = du.s;
   f.p_old = du.p_old;
@@ -167,6 +170,16 @@ pa_status fwd(pa_plan* p, const float* x, float* out, int mode, const void* y, c
   PA_CUDA(launch_forward(p->dim, f, st));
   PA_TRY(mark(t, true, st));
   return PA_OK;
+}
+
+// r = y - A x into the packed traces (and into r when not NULL), with the
+// partials of ||r||^2 in `parts`: residual_blocks() of them
+pa_status residual(pa_plan* p, const float* x, const void* y, float* r, float2* parts, Timing& t,
+                   cudaStream_t st) {
+  return fwd(p, x, r, FWD_RESID, y, stored(parts), t, st, DirUpdate(), true);
+}
+int residual_blocks(const pa_plan* p) {
+  return forward_combine_blocks(p->S, p->K, p->comb_spt, true);
 }
 
 pa_status adj(pa_plan* p, float* out, int mode, const double* omega, int nonneg,
@@ -214,8 +227,7 @@ pa_status enqueue_power(pa_plan* p, int n_pow, const float* v0, const Scalars& s
                       vec_blocks_r(N), st));
   PA_CUDA(launch_scale(p->d_pv, p->d_pv, sc.inv_lam, (int)N, st));
   for (int it = 0; it < n_pow; ++it) {
-    PA_TRY(fwd(p, p->d_pv, p->d_q, FWD_STORE, nullptr, none, t, st));
-    PA_CUDA(launch_pack(p->d_q, p->d_packed, p->S, p->K, p->Kp, p->pad, st));
+    PA_TRY(fwd(p, p->d_pv, nullptr, FWD_STORE, nullptr, none, t, st, DirUpdate(), true));
     PA_TRY(adj(p, p->d_sv, ADJ_NORM, nullptr, 0,
                make_reduce(p, OP_INVSQRT, sc.lam2, nullptr, sc.inv_lam), t, st));
     PA_CUDA(launch_scale(p->d_pv, p->d_sv, sc.inv_lam, (int)N, st));
@@ -234,13 +246,11 @@ pa_status enqueue_landweber(pa_plan* p, int n_iter, const void* y, float* x,
     omega = sc.inv_lam;
   }
   const Reduce none{};
-  const int n_comb = forward_combine_blocks(p->S, p->K, p->comb_spt);
+  const int n_comb = residual_blocks(p);
   for (int it = 0; it <= n_iter; ++it) {
     // r = y - A x; the partials of ||r||^2 go to history row it
-    PA_TRY(fwd(p, x, p->d_ra, FWD_RESID, y, stored(p->d_parts_h + (size_t)it * p->n_partials), t,
-               st));
+    PA_TRY(residual(p, x, y, nullptr, p->d_parts_h + (size_t)it * p->n_partials, t, st));
     if (it == n_iter) break;
-    PA_CUDA(launch_pack(p->d_ra, p->d_packed, p->S, p->K, p->Kp, p->pad, st));
     PA_TRY(adj(p, x, ADJ_LANDWEBER, omega, o.nonneg, none, t, st));  // x = max(0, x + w A^T r)
   }
   PA_CUDA(launch_hist(p->d_parts_h, p->n_partials, n_comb, n_comb, n_iter + 1, sc.hist, st));
@@ -258,12 +268,12 @@ pa_status enqueue_cgls(pa_plan* p, int n_iter, const void* y, float* x, const pa
   // (OP_STORE), the next kernel that needs the total sums them itself, and the
   // residual history is summed once after the loop (launch_hist).
   const int n_comb = forward_combine_blocks(p->S, p->K, p->comb_spt);
+  const int n_res = residual_blocks(p);
   const int n_adj = s_parts_count(p);  // partials of ||s||^2 (adj_norm)
   const int n_xr = cgls_r_blocks(p->S, p->K);
   float2* hist_row = p->d_parts_h;
   // r = y - A x0; s = A^T r; p = s (||r||^2 -> history row 0, ||s||^2 -> parts_s)
-  PA_TRY(fwd(p, x, r_in, FWD_RESID, y, stored(hist_row), t, st));
-  PA_CUDA(launch_pack(r_in, p->d_packed, p->S, p->K, p->Kp, p->pad, st));
+  PA_TRY(residual(p, x, y, r_in, hist_row, t, st));
   PA_TRY(adj_norm(p, p_cur, t, st));
   for (int it = 0; it < n_iter; ++it) {
     // p = s + beta p with beta = ||s||^2 / gamma (fused into the gather from the
@@ -303,7 +313,7 @@ pa_status enqueue_cgls(pa_plan* p, int n_iter, const void* y, float* x, const pa
     std::swap(r_in, r_out);
     std::swap(p_cur, p_prev);
   }
-  PA_CUDA(launch_hist(p->d_parts_h, p->n_partials, n_comb, n_xr, n_iter + 1, sc.hist, st));
+  PA_CUDA(launch_hist(p->d_parts_h, p->n_partials, n_res, n_xr, n_iter + 1, sc.hist, st));
   if (o.nonneg) PA_CUDA(launch_clamp(x, N, st));
   return PA_OK;
 }
@@ -315,14 +325,13 @@ pa_status enqueue_cgls(pa_plan* p, int n_iter, const void* y, float* x, const pa
 pa_status enqueue_pcgls(pa_plan* p, int n_iter, const void* y, float* x, const pa_recon_opts& o,
                         const Scalars& sc, Timing& t, cudaStream_t st) {
   const int N = p->grid.nx * p->grid.ny * p->grid.nz;
-  float* r = p->d_ra;
   float* p_cur = p->d_pv;
   float* p_prev = p->d_pb;
   const int n_comb = forward_combine_blocks(p->S, p->K, p->comb_spt);
+  const int n_res = residual_blocks(p);
   const int n_adj = s_parts_count(p);
   if (o.nonneg) PA_CUDA(launch_clamp(x, N, st));
-  PA_TRY(fwd(p, x, r, FWD_RESID, y, stored(p->d_parts_h), t, st));
-  PA_CUDA(launch_pack(r, p->d_packed, p->S, p->K, p->Kp, p->pad, st));
+  PA_TRY(residual(p, x, y, nullptr, p->d_parts_h, t, st));
   PA_TRY(adj_norm(p, p_cur, t, st));
   for (int it = 0; it < n_iter; ++it) {
     const int restart = o.restart > 0 && it % o.restart == 0;
@@ -354,20 +363,18 @@ pa_status enqueue_pcgls(pa_plan* p, int n_iter, const void* y, float* x, const p
     ca.gamma = sc.gamma + it;
     ca.delta = sc.delta + it;
     PA_CUDA(launch_cgls_x(x, p_cur, ca, N, p->S, p->K, o.nonneg, st));
-    PA_TRY(fwd(p, x, r, FWD_RESID, y, stored(p->d_parts_h + (size_t)(it + 1) * p->n_partials), t,
-               st));
-    PA_CUDA(launch_pack(r, p->d_packed, p->S, p->K, p->Kp, p->pad, st));
+    PA_TRY(residual(p, x, y, nullptr, p->d_parts_h + (size_t)(it + 1) * p->n_partials, t, st));
     PA_TRY(adj_norm(p, p->d_sv, t, st));
     std::swap(p_cur, p_prev);
   }
-  PA_CUDA(launch_hist(p->d_parts_h, p->n_partials, n_comb, n_comb, n_iter + 1, sc.hist, st));
+  PA_CUDA(launch_hist(p->d_parts_h, p->n_partials, n_res, n_res, n_iter + 1, sc.hist, st));
   return PA_OK;
 }
 
 // FISTA on F(x) = ||A x - y||^2 + alpha ||x||_1 + beta TV_eps(x) (Eq. 8 with
-// Phi = A, Psi' = I): per iteration r = y - A z (||r||^2 -> history), the TV
-// gradient at z, then A^T r with the proximal step and the extrapolation in the
-// adjoint's epilogue.  The momentum weights (t_k - 1)/t_{k+1} depend on k only
+// Phi = A, Psi' = I): per iteration r = y - A z (||r||^2 -> history), then A^T r
+// with the TV gradient at z, the proximal step and the extrapolation in the
+// adjoint's epilogue (z ping-pongs: the gradient reads neighbours of z).  The momentum weights (t_k - 1)/t_{k+1} depend on k only
 // and are baked into the launches.
 pa_status enqueue_fista(pa_plan* p, int n_iter, const void* y, float* x, const pa_recon_opts& o,
                         const Scalars& sc, Timing& t, cudaStream_t st) {
@@ -379,21 +386,17 @@ pa_status enqueue_fista(pa_plan* p, int n_iter, const void* y, float* x, const p
     PA_CUDA(launch_fista_tau(sc.omega, sc.inv_lam, 8.0 * o.tv_weight / o.tv_eps, st));
   }
   float* z = p->d_pv;
-  float* tvg = p->d_sv;
+  float* z_next = p->d_pb;
   PA_CUDA(cudaMemcpyAsync(z, x, (size_t)N * sizeof(float), cudaMemcpyDeviceToDevice, st));
-  const int n_comb = forward_combine_blocks(p->S, p->K, p->comb_spt);
+  const int n_comb = residual_blocks(p);
   double tk = 1.0;
   for (int it = 0; it < n_iter; ++it) {
-    PA_TRY(fwd(p, z, p->d_ra, FWD_RESID, y, stored(p->d_parts_h + (size_t)it * p->n_partials), t,
-               st));
-    PA_CUDA(launch_pack(p->d_ra, p->d_packed, p->S, p->K, p->Kp, p->pad, st));
-    if (o.tv_weight != 0.0)
-      PA_CUDA(launch_tv(p->dim, z, p->grid.nx, p->grid.ny, p->grid.nz, (float)o.tv_eps, tvg,
-                        stored(p->d_parts_q), st));
+    PA_TRY(residual(p, z, y, nullptr, p->d_parts_h + (size_t)it * p->n_partials, t, st));
     const double tn = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * tk * tk));
     AdjParams a = adjoint_params(p, x, ADJ_FISTA, sc.omega, o.nonneg);
     a.z = z;
-    a.tvg = o.tv_weight != 0.0 ? tvg : z;  // unused when tv_beta = 0
+    a.z_out = z_next;
+    a.tv_eps2 = (float)o.tv_eps * (float)o.tv_eps;
     a.l1 = (float)o.l1_weight;
     a.tv_beta = (float)o.tv_weight;
     a.mu = (float)((tk - 1.0) / tn);
@@ -401,9 +404,9 @@ pa_status enqueue_fista(pa_plan* p, int n_iter, const void* y, float* x, const p
     PA_CUDA(launch_adjoint(p->dim, a, p->cluster, p->ntiles, st));
     PA_TRY(mark(t, false, st));
     tk = tn;
+    std::swap(z, z_next);
   }
-  PA_TRY(fwd(p, x, p->d_ra, FWD_RESID, y,
-             stored(p->d_parts_h + (size_t)n_iter * p->n_partials), t, st));
+  PA_TRY(residual(p, x, y, nullptr, p->d_parts_h + (size_t)n_iter * p->n_partials, t, st));
   PA_CUDA(launch_hist(p->d_parts_h, p->n_partials, n_comb, n_comb, n_iter + 1, sc.hist, st));
   return PA_OK;
 }
@@ -668,8 +671,7 @@ pa_status pa_shard_cgls_begin(pa_plan* plan, int n_iter, const void* y_dev, cons
   Timing none;
   float* r0 = shard_r(plan, 0);
   // r_0 = y - A x_0 (||r_0||^2 -> history row 0); s_part = A^T r_0
-  PA_TRY(fwd(plan, x_dev, r0, FWD_RESID, y_dev, stored(plan->d_parts_h), none, st));
-  PA_CUDA(launch_pack(r0, plan->d_packed, plan->S, plan->K, plan->Kp, plan->pad, st));
+  PA_TRY(residual(plan, x_dev, y_dev, r0, plan->d_parts_h, none, st));
   PA_TRY(shard_adjoint(plan, s_part_dev, accumulate, st));
   plan->shard_n = n_iter;
   plan->shard_it = 0;
@@ -769,9 +771,8 @@ pa_status pa_shard_cgls_finish(pa_plan* plan, float* x_dev, int nonneg, double* 
   cudaStream_t st = (cudaStream_t)stream;
   const int n_done = plan->shard_it;
   if (hist_dev) {
-    const int n_comb = forward_combine_blocks(plan->S, plan->K, plan->comb_spt);
     const int n_xr = cgls_r_blocks(plan->S, plan->K);
-    PA_CUDA(launch_hist(plan->d_parts_h, plan->n_partials, n_comb, n_xr, n_done + 1, hist_dev, st,
+    PA_CUDA(launch_hist(plan->d_parts_h, plan->n_partials, residual_blocks(plan), n_xr, n_done + 1, hist_dev, st,
                         accumulate ? 1 : 0));
   }
   if (nonneg) PA_CUDA(launch_clamp(x_dev, plan->grid.nx * plan->grid.ny * plan->grid.nz, st));
