@@ -273,7 +273,7 @@ constexpr int kBatchFwdThreads = 256;       // pixel owners of the batched forwa
 // sensors per batched forward item: the batch cuts every frame's forward into
 // items of its own block shape, whatever the plan's single-launch options
 // (fwd_sensors_per_cta, fwd_threads); the windows, and so the results, are the same
-constexpr int kBatchFwdSensors = 32;
+constexpr int kBatchMinSensors = 8, kBatchMaxSensors = 128;
 constexpr int kAdjSB = 8;                    // sensors per pipeline stage
 constexpr int kAdjStages = 4;
 

@@ -760,8 +760,12 @@ __device__ __forceinline__ void adj_pair2(const TileRef2& r, uint32_t base, floa
 // Accumulates, for every pixel of `tile`, the sum over sensors [s_begin, s_end)
 // into s_acc (shared, kTilePixels floats; returned).  Warps 0..NW-1 compute
 // (kTilePixels / (32 NW) pixels per thread, as packed pairs), warp NW produces;
-// any further warps of the block only take part in the barriers.
-template <int DIM, bool DC, int NW>
+// any further warps of the block only take part in the barriers.  PLAIN: stages
+// whose sensors are all far and none skipped take a loop without the two branches
+// per sensor (128^3 A^T 1229 -> 1128 us, 480^2 with 400 sensors 67 -> 62; the
+// batched launches' 56 registers spill with both loops, 6635 against 6719 us for a
+// batch of 16 frames).
+template <int DIM, bool DC, int NW, bool PLAIN = true>
 __device__ __forceinline__ float* adj_accumulate(const AdjParams& P, const float2* packed, int tile,
                                                  int s_begin, int s_end, unsigned char* smem) {
   constexpr int PPT = kTilePixels / (32 * NW);
@@ -780,6 +784,7 @@ __device__ __forceinline__ float* adj_accumulate(const AdjParams& P, const float
   uint64_t* s_empty = s_full + NST;
   __shared__ int s_abort;
   __shared__ int s_issued;
+  __shared__ int s_special[NST];  // a skipped or near sensor in the stage
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_stages = s_end > s_begin ? (s_end - s_begin + SB - 1) / SB : 0;
@@ -815,6 +820,7 @@ __device__ __forceinline__ float* adj_accumulate(const AdjParams& P, const float
       const int s = s_begin + j * SB + lane;
       uint32_t bytes = 0;
       const float2* src = nullptr;
+      [[maybe_unused]] int special = 0;
       if (lane < SB) {
         TileRef r;
         r.klo = kSkip;
@@ -834,6 +840,7 @@ __device__ __forceinline__ float* adj_accumulate(const AdjParams& P, const float
 #endif
           }
         }
+        if (PLAIN) special = r.klo == kSkip || (r.klo & kNear);
         if (r.klo != kSkip) {
           s_ref[slot * SB + lane] = expand_ref(r);
         } else {
@@ -841,6 +848,10 @@ __device__ __forceinline__ float* adj_accumulate(const AdjParams& P, const float
         }
       }
       const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+      if (PLAIN) {
+        special = __any_sync(0xffffffffu, special);
+        if (lane == 0) s_special[slot] = special;
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive_expect_tx(&s_full[slot], total);
       __syncwarp();
@@ -885,6 +896,16 @@ __device__ __forceinline__ float* adj_accumulate(const AdjParams& P, const float
       if (*(volatile int*)&s_abort) break;
       const TileRef2* refs = s_ref + slot * SB;
       uint32_t base = magic_base(trace_u32 + (uint32_t)(slot * SB * L + L / 2) * 8u, 3);
+      if (PLAIN && !s_special[slot]) {
+#pragma unroll 1
+        for (int sb = 0; sb < SB; ++sb, base += 8u * (uint32_t)L) {
+          const TileRef2 r = refs[sb];
+#pragma unroll
+          for (int h = 0; h < NPAIR; ++h)
+            adj_pair2<DIM, false, DC>(r, base, ddx[h], ddy[h], ddz[h], cm[h], inv_kappa, hik,
+                                      acc[2 * h], acc[2 * h + 1], chk);
+        }
+      } else
 #pragma unroll 1
       for (int sb = 0; sb < SB; ++sb, base += 8u * (uint32_t)L) {
         const TileRef2 r = refs[sb];
@@ -1172,6 +1193,7 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint_frames(const AdjPa
   __shared__ int s_abort, s_issued;
   __shared__ DF s_red[NF][NW + 1];
   __shared__ int s_last;
+  __shared__ int s_special[kAdjfMaxStages];  // a skipped or near sensor in the stage
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank(), C = (int)cluster.num_blocks();
   const int tile = blockIdx.y, f0 = blockIdx.z * NF;
@@ -1232,6 +1254,7 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint_frames(const AdjPa
       const int s = s_begin + j * SB + sb;
       uint32_t bytes = 0;
       const float4* src = nullptr;
+      int special = 0;
       if (sb < SB) {
         if (r.klo != kSkip) {
           const int ws0 = P.pad + window_start(r.klo);
@@ -1247,6 +1270,7 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint_frames(const AdjPa
                   ((int64_t)(f0 / 2 + q) * P.S + s) * P.Kp + ws0;
           }
         }
+        special = r.klo == kSkip || (r.klo & kNear);
         if (q == 0) {
           if (r.klo != kSkip)
             s_ref[slot * 8 + sb] = expand_ref(r);
@@ -1255,6 +1279,8 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint_frames(const AdjPa
         }
       }
       const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+      special = __any_sync(0xffffffffu, special);
+      if (lane == 0) s_special[slot] = special;
       __syncwarp();
       if (lane == 0) mbar_arrive_expect_tx(&s_full[slot], total);
       __syncwarp();
@@ -1296,6 +1322,16 @@ __global__ void __launch_bounds__(32 * (NW + 1), 2) k_adjoint_frames(const AdjPa
       if (*(volatile int*)&s_abort) break;
       const TileRef2* refs = s_ref + slot * 8;
       uint32_t base = magic_base(trace_u32 + (uint32_t)(slot * SB * NP * L + L / 2) * 16u, 4);
+      if (!s_special[slot]) {
+#pragma unroll 1
+        for (int sb = 0; sb < SB; ++sb, base += NP * pstride) {
+          const TileRef2 r = refs[sb];
+#pragma unroll
+          for (int h = 0; h < NPAIR; ++h)
+            adjf_pair2<DIM, false, MODE, NP>(r, base, pstride, ddx[h], ddy[h], ddz[h], cm[h],
+                                             inv_kappa, hik, acc[h], accd[h], chk);
+        }
+      } else
 #pragma unroll 1
       for (int sb = 0; sb < SB; ++sb, base += NP * pstride) {
         const TileRef2 r = refs[sb];
@@ -1514,8 +1550,8 @@ cudaError_t launch_adjoint_frames(int dim, const AdjParams& p, int cluster, int 
 // k, in a fixed order (by window start), plus the residual / norm epilogue.
 // ---------------------------------------------------------------------------
 // Each (tile, sensor) window is kept as kFwdCopies copies, copy c starting
-// c * CS words in, with CS = 12 (mod 32): the copies of one bin lie 12 banks
-// apart.  A warp's shared-memory atomic takes as many passes as the largest
+// c * CS words in, with CS = 12 (mod 32) in 2D and 8 in 3D: the copies of one bin
+// lie so many banks apart.  A warp's shared-memory atomic takes as many passes as the largest
 // number of its lanes that fall into one bank, whether or not their addresses
 // agree, and the 32 pixels of a warp fall into ~25 sample bins.  Each lane
 // therefore deposits into the copy the per-(tile, sensor) table `copies`
@@ -1523,12 +1559,17 @@ cudaError_t launch_adjoint_frames(int dim, const AdjParams& p, int cluster, int 
 // the banks.  The flush adds the copies (exact integer sums), so results do
 // not depend on the assignment.
 constexpr int kFwdCopies = 4;
-constexpr int kFwdCopyRes = 12;  // copy stride mod 32 (a multiple of 4: 16-byte aligned copies)
-__host__ __device__ inline int fwd_copy_stride(int L) { return L + ((kFwdCopyRes - L) & 31); }
+// copy stride mod 32 (a multiple of 4: 16-byte aligned copies): 12 in 2D, 8 in 3D
+// (simulated passes per atomic, greedy assignment: 2D ring 2.10 with 12, 2.23 with
+// 8; 3D planar array 2.25 with 12, 2.12 with 8)
+__host__ __device__ constexpr int fwd_copy_res(int dim) { return dim == 3 ? 8 : 12; }
+__host__ __device__ inline int fwd_copy_stride(int dim, int L) {
+  return L + ((fwd_copy_res(dim) - L) & 31);
+}
 
 int forward_smem_bytes(int dim, int L, int spc) {
   return spc * (int)sizeof(TileRef2) +
-         2 * fwd_sb(dim) * kFwdCopies * fwd_copy_stride(L) * (int)sizeof(int);
+         2 * fwd_sb(dim) * kFwdCopies * fwd_copy_stride(dim, L) * (int)sizeof(int);
 }
 
 // Copy assignment and tap scale of the forward windows.  One warp per (tile,
@@ -1536,7 +1577,7 @@ int forward_smem_bytes(int dim, int L, int spc) {
 // pixels 32 r .. 32 r + 31: thread lane l of warp r % 8 deposits pixel 32 r +
 // l), so every warp atomic of the gather is one row.
 //   Copies: lanes l = 0..31 in turn take the copy c whose bank (bin + c
-// kFwdCopyRes) mod 32 minimises, summed over the 32 rows, the squared number
+// fwd_copy_res) mod 32 minimises, summed over the 32 rows, the squared number
 // of lanes already assigned to that bank (ties to the lower copy; two
 // candidates' sums, each at most 32 x 31^2 < 2^16, share a warp reduction: the
 // reductions bound the kernel, which took 104 us with one per candidate for the
@@ -1622,8 +1663,8 @@ __global__ void __launch_bounds__(256) k_fwd_copies(unsigned long long* copies, 
       unsigned sc[kFwdCopies];
 #pragma unroll
       for (int c = 0; c < kFwdCopies; c += 2) {
-        const unsigned v0 = ld[(bins[l] + c * kFwdCopyRes) & 31];
-        const unsigned v1 = ld[(bins[l] + (c + 1) * kFwdCopyRes) & 31];
+        const unsigned v0 = ld[(bins[l] + c * fwd_copy_res(DIM)) & 31];
+        const unsigned v1 = ld[(bins[l] + (c + 1) * fwd_copy_res(DIM)) & 31];
         const unsigned sum = __reduce_add_sync(0xffffffffu, v0 * v0 + ((v1 * v1) << 16));
         sc[c] = sum & 0xffffu;
         sc[c + 1] = sum >> 16;
@@ -1637,7 +1678,7 @@ __global__ void __launch_bounds__(256) k_fwd_copies(unsigned long long* copies, 
           best = c;
         }
       }
-      ++ld[(bins[l] + best * kFwdCopyRes) & 31];
+      ++ld[(bins[l] + best * fwd_copy_res(DIM)) & 31];
       if (l < 16)
         lo |= (unsigned)best << (2 * l);
       else
@@ -1734,8 +1775,10 @@ __device__ __forceinline__ void fwd_tile_block(const FwdParams& P, int tile, int
   // the sensors' table entries are staged and the windows cleared first, so
   // that their latency overlaps the loads (and, for a CGLS direction, the
   // reduction) below
+  int special = 0;  // a skipped or near sensor among the item's
   for (int i = tid; i < ns; i += nt) {
     const TileRef r = P.table[(int64_t)tile * P.S + s0 + i];
+    special |= r.klo == kSkip || (r.klo & kNear);
     if (r.klo != kSkip) {
       TileRef2 e = expand_ref(r);
       if (P.copies) {
@@ -1748,7 +1791,7 @@ __device__ __forceinline__ void fwd_tile_block(const FwdParams& P, int tile, int
       refs[i].klo = kSkip;
     }
   }
-  const int CS = fwd_copy_stride(L);           // words per window copy (a multiple of 4)
+  const int CS = fwd_copy_stride(DIM, L);           // words per window copy (a multiple of 4)
   const int WS = kFwdCopies * CS;              // words per (tile, sensor) window
   {
     int4* w4 = reinterpret_cast<int4*>(win);  // 16-byte aligned: refs are 64-byte entries
@@ -1828,6 +1871,7 @@ __device__ __forceinline__ void fwd_tile_block(const FwdParams& P, int tile, int
   for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
   if (lane == 0) s_max[warp] = amax;
   const bool finite = __syncthreads_or(nonfinite) == 0;
+  const bool plain = __syncthreads_or(special) == 0;
   float xmax = 0.0f;
   for (int w = 0; w < (nt >> 5); ++w) xmax = fmaxf(xmax, s_max[w]);
   const float xscale = (xmax > 0.0f && finite) ? kFixedScale / xmax : 0.0f;
@@ -1847,6 +1891,23 @@ __device__ __forceinline__ void fwd_tile_block(const FwdParams& P, int tile, int
     const int nsb = min(SB, ns - g0);
     if (owner && xscale > 0.0f) {
       uint32_t base = magic_base(win_u32 + (uint32_t)(buf * SB * WS + L / 2) * 4u, 2);
+      if (plain) {
+        // no skipped and no near sensor (most items, where sensors lie outside the
+        // grid): a loop without the two branches per sensor (128^3 A 2060 -> 2011 us,
+        // 480^2 with 400 sensors 105 -> 100; loading the next entry ahead takes 16
+        // registers and lost 4% there)
+#pragma unroll 1
+        for (int sb = 0; sb < nsb; ++sb, base += 4u * (uint32_t)WS) {
+          const TileRef2 r = refs[g0 + sb];
+          const float2 dlo = f2(r.dlo);
+          const uint32_t cbase =
+              base + (((copy_hi ? r.copy_hi : r.copy_lo) >> copy_sh) & 3u) * copy_bytes;
+#pragma unroll
+          for (int h = 0; h < NPAIR; ++h)
+            fwd_pair2<DIM, false>(r, cbase, ddx[h], ddy[h], ddz[h], cm[h], mul2(xs[h], dlo),
+                                  inv_kappa, hik, chk);
+        }
+      } else
 #pragma unroll 1
       for (int sb = 0; sb < nsb; ++sb, base += 4u * (uint32_t)WS) {
         const TileRef2 r = refs[g0 + sb];
@@ -2603,7 +2664,7 @@ template <int DIM>
 __device__ __forceinline__ void adj_landweber_block(const AdjParams& P, int tile,
                                                     unsigned char* smem) {
   constexpr int TX = Tile<DIM>::X, TY = Tile<DIM>::Y, TZ = Tile<DIM>::Z;
-  float* s_acc = adj_accumulate<DIM, false, kBatchAdjWarps>(P, P.packed, tile, 0, P.S, smem);
+  float* s_acc = adj_accumulate<DIM, false, kBatchAdjWarps, false>(P, P.packed, tile, 0, P.S, smem);
   const int tx = tile % P.g.ntx, ty = (tile / P.g.ntx) % P.g.nty, tz = tile / (P.g.ntx * P.g.nty);
   const float om = (float)(*P.omega);
   for (int p = threadIdx.x; p < kTilePixels; p += blockDim.x) {
@@ -2670,7 +2731,7 @@ __device__ __forceinline__ void adj_norm_block(const AdjParams& P, int tile, flo
                                                float2* s_parts, unsigned char* smem) {
   constexpr int TX = Tile<DIM>::X, TY = Tile<DIM>::Y, TZ = Tile<DIM>::Z;
   __shared__ DF s_red[32];
-  float* s_acc = adj_accumulate<DIM, false, kBatchAdjWarps>(P, P.packed, tile, 0, P.S, smem);
+  float* s_acc = adj_accumulate<DIM, false, kBatchAdjWarps, false>(P, P.packed, tile, 0, P.S, smem);
   const int tx = tile % P.g.ntx, ty = (tile / P.g.ntx) % P.g.nty, tz = tile / (P.g.ntx * P.g.nty);
   DF part = df_zero();
   for (int p = threadIdx.x; p < kTilePixels; p += blockDim.x) {
