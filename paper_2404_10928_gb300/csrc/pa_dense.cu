@@ -11,8 +11,14 @@
 // (pixel, sensor) pair are non-zero, so assembly is a zero fill plus one
 // thread per pair writing its two entries, evaluated in FP64 with the
 // oracle's operation order (no FMA contraction) and rounded once for FP32.
-// The products are bound by HBM (one pass over M) or, in FP64, by GB300's FP64
-// pipe (one FMA per entry at ~1/64 of the FP32 rate); every sum runs in a
+// The products are bound by HBM (one pass over M).  In FP64 one FMA per entry would
+// bind them to GB300's FP64 pipe (~64 cycles per warp instruction: 189 and 182 us at
+// 6144 x 16384, against 118 us for the bytes at 6.8 TB/s); a measurement matrix is
+// mostly zeros (two entries per pixel and sensor), so a round of entries that are
+// all zero for a warp and meet finite vector values, which would leave the sums as
+// they are, is skipped on integer tests: both products together 374 -> 255 us (237 for
+// the bytes).  Every entry of a full matrix costs the tests besides.  (Skipped one by
+// one, the FMAs are predicated and still take their turn in the pipe.)  Every sum runs in a
 // fixed order, so results are bitwise reproducible.
 #include "pa_internal.cuh"
 
@@ -49,6 +55,13 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_taps(
   const int64_t k = (int64_t)k0;
   if (k >= 0 && k < K) m[((int64_t)s * K + k) * cols + i] = (T)__dmul_rn(w, __dsub_rn(1.0, f));
   if (k + 1 >= 0 && k + 1 < K) m[((int64_t)s * K + k + 1) * cols + i] = (T)__dmul_rn(w, f);
+}
+
+// Whether a product a b can change a sum that started at +0 (and so never is -0):
+// a is not +-0, or b is infinite or NaN.  Integer tests keep off the FP64 pipe.
+__device__ __forceinline__ bool counts(double a, double b) {
+  return ((__double2hiint(a) << 1) | __double2loint(a)) != 0 ||
+         (__double2hiint(b) & 0x7ff00000) == 0x7ff00000;
 }
 
 template <typename T>
@@ -98,6 +111,12 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_mv(const T* m, const T*
         a[u] = __ldcs(rv + j + u * kDenseThreads);
         b[u] = __ldg(vv + j + u * kDenseThreads);
       }
+      if constexpr (sizeof(T) == 8) {
+        bool any = false;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) any |= counts(a[u].x, b[u].x) | counts(a[u].y, b[u].y);
+        if (!__any_sync(__activemask(), any)) continue;
+      }
 #pragma unroll
       for (int u = 0; u < 4; ++u) dot(a[u], b[u]);
     }
@@ -127,7 +146,27 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_mtv(const T* m, const T
   const int64_t r1 = min(rows, r0 + kRowsPerChunk);
   if (c < cols) {
     T acc = 0;
-    for (int64_t r = r0; r < r1; ++r) acc += __ldcs(m + r * cols + c) * __ldg(v + r);
+    if constexpr (sizeof(T) == 8) {
+      // rounds of eight rows, loaded before the tests decide
+      constexpr int U = 8;
+      for (int64_t r = r0; r < r1; r += U) {
+        T a[U], b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const bool in = r + u < r1;
+          a[u] = in ? __ldcs(m + (r + u) * cols + c) : T(0);
+          b[u] = in ? __ldg(v + r + u) : T(0);
+        }
+        bool any = false;
+#pragma unroll
+        for (int u = 0; u < U; ++u) any |= counts(a[u], b[u]);
+        if (!__any_sync(__activemask(), any)) continue;
+#pragma unroll
+        for (int u = 0; u < U; ++u) acc = fma(a[u], b[u], acc);  // absent rows add +0
+      }
+    } else {
+      for (int64_t r = r0; r < r1; ++r) acc += __ldcs(m + r * cols + c) * __ldg(v + r);
+    }
     part[(int64_t)blockIdx.y * cols + c] = acc;
   }
   __threadfence();
