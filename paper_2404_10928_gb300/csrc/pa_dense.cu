@@ -17,7 +17,7 @@
 // mostly zeros (two entries per pixel and sensor), so a round of entries that are
 // all zero for a warp and meet finite vector values, which would leave the sums as
 // they are, is skipped on integer tests: both products together 374 -> 255 us (237 for
-// the bytes).  Every entry of a full matrix costs the tests besides.  (Skipped one by
+// the bytes).  A matrix without zeros pays the tests (190 to 191 and 183 to 188 us).  (Skipped one by
 // one, the FMAs are predicated and still take their turn in the pipe.)  Every sum runs in a
 // fixed order, so results are bitwise reproducible.
 #include "pa_internal.cuh"
@@ -149,21 +149,22 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_mtv(const T* m, const T
     if constexpr (sizeof(T) == 8) {
       // rounds of eight rows, loaded before the tests decide
       constexpr int U = 8;
-      for (int64_t r = r0; r < r1; r += U) {
+      int64_t r = r0;
+      for (; r + U <= r1; r += U) {
         T a[U], b[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const bool in = r + u < r1;
-          a[u] = in ? __ldcs(m + (r + u) * cols + c) : T(0);
-          b[u] = in ? __ldg(v + r + u) : T(0);
+          a[u] = __ldcs(m + (r + u) * cols + c);
+          b[u] = __ldg(v + r + u);
         }
         bool any = false;
 #pragma unroll
         for (int u = 0; u < U; ++u) any |= counts(a[u], b[u]);
         if (!__any_sync(__activemask(), any)) continue;
 #pragma unroll
-        for (int u = 0; u < U; ++u) acc = fma(a[u], b[u], acc);  // absent rows add +0
+        for (int u = 0; u < U; ++u) acc = fma(a[u], b[u], acc);
       }
+      for (; r < r1; ++r) acc = fma(__ldcs(m + r * cols + c), __ldg(v + r), acc);
     } else {
       for (int64_t r = r0; r < r1; ++r) acc += __ldcs(m + r * cols + c) * __ldg(v + r);
     }
