@@ -63,10 +63,10 @@ def cores():
 
 def cgls_launches(n_iter: int) -> int:
     """Kernels of one CGLS reconstruction (A = tile gather + combine; every norm
-    is summed by the kernel that consumes it): setup (A, pack, A^T) = 4, per
-    iteration (A with the fused direction update, alpha + x/r update, A^T) = 4,
-    then the residual history and the final clamp = 2."""
-    return 4 + 4 * n_iter + 2
+    is summed by the kernel that consumes it): setup (A with its packed residual,
+    A^T) = 3, per iteration (A with the fused direction update, alpha + x/r
+    update, A^T) = 4, then the residual history and the final clamp = 2."""
+    return 3 + 4 * n_iter + 2
 
 
 def max_over_ranks(dist, device, value: float) -> float:
