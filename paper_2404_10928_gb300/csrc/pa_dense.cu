@@ -16,10 +16,10 @@
 // 6144 x 16384, against 118 us for the bytes at 6.8 TB/s); a measurement matrix is
 // mostly zeros (two entries per pixel and sensor), so a round of entries that are
 // all zero for a warp and meet finite vector values, which would leave the sums as
-// they are, is skipped on integer tests: both products together 374 -> 255 us (237 for
-// the bytes).  A matrix without zeros pays the tests (190 to 191 and 183 to 188 us).  (Skipped one by
-// one, the FMAs are predicated and still take their turn in the pipe.)  Every sum runs in a
-// fixed order, so results are bitwise reproducible.
+// they are, is skipped on integer tests: both products together 374 -> 255 us (237
+// for the bytes).  A matrix without zeros pays the tests (190 to 191 and 183 to 188
+// us).  (Skipped one by one, the FMAs are predicated and still take their turn in
+// the pipe.)  Every sum runs in a fixed order, so results are bitwise reproducible.
 #include "pa_internal.cuh"
 
 namespace pa {
