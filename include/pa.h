@@ -91,7 +91,7 @@ typedef struct {
  *               1024 / fwd_threads pixels of the tile (0 = 128).
  *   adj_warps    compute warps per adjoint CTA: 4 or 8, each thread owning
  *               1024 / (32 adj_warps) pixels of the tile (0 = chosen from the
- *               dimension and adj_cluster).
+ *               dimension, adj_cluster and sensors).
  * The last four are the tile shapes an autotuner may pick; none changes a
  * result bit of the forward (its window sums are exact integer sums), and
  * adj_warps none of the adjoint's image (each pixel sums its sensors in

@@ -326,7 +326,7 @@ pa_status validate_grid(const pa_grid* g);
 // the gathers' work split where the caller leaves it open (pa_plan.cu)
 int default_fwd_sensors(int64_t units, int sms);
 int default_cluster(int dim, int64_t ntiles, int S, int sms);
-int default_adj_warps(int dim, int cluster);
+int default_adj_warps(int dim, int cluster, int S);
 
 // reductions and vector updates
 cudaError_t launch_cgls_xr(float* x, const float* pvec, const float* r_in, float* r_out,

@@ -85,11 +85,14 @@ int default_cluster(int dim, int64_t ntiles, int S, int sms) {
   return C;
 }
 
-// Compute warps of an adjoint CTA: four (eight pixels per thread) where a cluster
-// gives each CTA few sensors (2D: 64 tiles, 256 sensors 20.5 -> 18.5 us, 144 tiles,
-// 200 sensors 28.3 -> 26.6); eight otherwise (the same within 1% at two CTAs per
-// tile; 128^3 1260 against 1230 us).
-int default_adj_warps(int dim, int cluster) { return dim == 2 && cluster >= 4 ? 4 : 8; }
+// Compute warps of an adjoint CTA: four (eight pixels per thread) where clusters are
+// large (2D: 64 tiles, 256 sensors 20.5 -> 18.5 us, 144 tiles, 200 sensors 28.3 ->
+// 26.6); eight otherwise (the same within 1% at two CTAs per tile; 128^3 1260 against
+// 1230 us) and where a CTA has fewer than 16 sensors (64^2 with 64 sensors: 8.2 us
+// with either).
+int default_adj_warps(int dim, int cluster, int S) {
+  return dim == 2 && cluster >= 4 && S >= 16 * cluster ? 4 : 8;
+}
 
 // Sensors per forward work item: about 800 items where there is little work
 // (64^2, 64 sensors: 13.3 us with 8 sensors per item, 20.5 with 32; 301 x 187, 173
@@ -374,7 +377,7 @@ pa_status pa_plan_create(pa_plan** out, const double* sensors_xyz, int n_sensors
     p->cluster = default_cluster(p->dim, p->ntiles, p->S, sms);
     if (opts && opts->adj_cluster > 0) p->cluster = std::min(opts->adj_cluster, p->S);
     p->adj_warps = opts && opts->adj_warps > 0 ? opts->adj_warps
-                                               : default_adj_warps(p->dim, p->cluster);
+                                               : default_adj_warps(p->dim, p->cluster, p->S);
     p->fwd_spc = default_fwd_sensors((int64_t)p->ntiles * p->S, sms);
     if (forward_smem_bytes(p->dim, p->L, p->fwd_spc) > 200 * 1024)
       p->fwd_spc = std::min(p->fwd_spc, kFwdSPC);
