@@ -120,6 +120,13 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
+// Orders this thread's ordinary (generic-proxy) reads and writes of global and
+// shared memory against bulk copies (async proxy) on the other side of it.  A
+// __threadfence or a barrier alone does not order the two proxies.
+__device__ __forceinline__ void fence_proxy_async() {
+  asm volatile("fence.proxy.async;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Reductions in double-float arithmetic (an unevaluated FP32 pair hi + lo,
 // Dekker 1971; TwoSum of Knuth, TAOCP vol. 2, Sec. 4.2.2).  GB300's FP64 pipe
@@ -2621,9 +2628,16 @@ cudaError_t launch_tv_frames(int dim, const float* x, int nx, int ny, int nz, fl
 // on (the result is then invalid, but the launch ends).
 // state: [0] arrivals, [1] generation, [2] forward queue, [3] combine queue,
 // [4] adjoint queue.
+//   to_bulk: the next phase reads with bulk copies what this and earlier phases
+// wrote with ordinary stores (the packed traces, by any CTA), into shared memory
+// that they used (the forward's windows): every writing thread fences the proxies
+// before the barrier and every thread that may issue a copy after it.  Separate
+// launches need neither.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void grid_barrier(unsigned* st, unsigned nblocks, int* err,
-                                             unsigned* queue_to_reset, uint64_t wait_ns) {
+                                             unsigned* queue_to_reset, uint64_t wait_ns,
+                                             bool to_bulk = false) {
+  if (to_bulk) fence_proxy_async();
   __syncthreads();
   if (threadIdx.x == 0) {
     volatile unsigned* gen = st + 1;
@@ -2652,6 +2666,7 @@ __device__ __forceinline__ void grid_barrier(unsigned* st, unsigned nblocks, int
     __threadfence();
   }
   __syncthreads();
+  if (to_bulk) fence_proxy_async();
 }
 
 __device__ __forceinline__ int grab_item(unsigned* queue) {
@@ -2718,7 +2733,7 @@ __global__ void __launch_bounds__(kBatchThreads, 4) k_batch_landweber(
       const int nk = frames[f].n_kblk;
       combine_block<FWD_RESID, 4, true>(P, li / nk, li % nk, nk);
     }
-    grid_barrier(state, nb, err, state + 3, wait_ns);
+    grid_barrier(state, nb, err, state + 3, wait_ns, true);
     if (it == n_iter) break;
     for (int gi = grab_item(state + 4); gi < pa[nf]; gi = grab_item(state + 4)) {
       const int f = frame_of(pa, nf, gi);
@@ -2797,7 +2812,7 @@ __global__ void __launch_bounds__(kBatchThreads, 4) k_batch_cgls(
     const int nk = frames[f].n_kblk;
     combine_block<FWD_RESID, 4, true>(P, li / nk, li % nk, nk);
   }
-  grid_barrier(state, nb, err, state + 3, wait_ns);
+  grid_barrier(state, nb, err, state + 3, wait_ns, true);
   for (int gi = grab_item(state + 4); gi < pa[nf]; gi = grab_item(state + 4)) {
     const int f = frame_of(pa, nf, gi);
     adj_norm_block<DIM>(frames[f].a, gi - pa[f], frames[f].pbuf[0], frames[f].s_parts, smem);
@@ -2855,7 +2870,7 @@ __global__ void __launch_bounds__(kBatchThreads, 4) k_batch_cgls(
                                      stored_parts(B.h_parts + (int64_t)(it + 1) * B.h_stride), li,
                                      B.n_xr);
     }
-    grid_barrier(state, nb, err, state + 5, wait_ns);
+    grid_barrier(state, nb, err, state + 5, wait_ns, true);
     // s = A^T r (||s||^2 per tile)
     for (int gi = grab_item(state + 4); gi < pa[nf]; gi = grab_item(state + 4)) {
       const int f = frame_of(pa, nf, gi);
