@@ -40,6 +40,9 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
                : "memory");
 }
+__device__ __forceinline__ void mbar_inval(uint64_t* bar) {
+  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -771,7 +774,7 @@ __device__ __forceinline__ void adj_pair2(const TileRef2& r, uint32_t base, floa
 // whose sensors are all far and none skipped take a loop without the two branches
 // per sensor (128^3 A^T 1229 -> 1128 us, 480^2 with 400 sensors 67 -> 62; the
 // batched launches' 56 registers spill with both loops, 6635 against 6719 us for a
-// batch of 16 frames).
+// batch of 16 frames).  !PLAIN: a CTA may call it again.
 template <int DIM, bool DC, int NW, bool PLAIN = true>
 __device__ __forceinline__ float* adj_accumulate(const AdjParams& P, const float2* packed, int tile,
                                                  int s_begin, int s_end, unsigned char* smem) {
@@ -959,7 +962,14 @@ __device__ __forceinline__ float* adj_accumulate(const AdjParams& P, const float
     for (int jj = max(0, issued - NST); jj < issued; ++jj)
       mbar_wait_bounded(&s_full[jj % NST], (jj / NST) & 1);
   }
-
+  if (!PLAIN && tid == 0) {
+    // a persistent launch uses this memory again: for the forward's windows, and
+    // for the next item's barriers (no thread waits on these any more)
+    for (int i = 0; i < NST; ++i) {
+      mbar_inval(&s_full[i]);
+      mbar_inval(&s_empty[i]);
+    }
+  }
   __syncthreads();
   return s_acc;
 }

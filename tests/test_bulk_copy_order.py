@@ -45,3 +45,15 @@ def test_adjoint_phases_follow_a_fenced_barrier(kernel):
     for before, (_, adj) in zip(events, events[1:]):
         if adj:
             assert before[0] and before[0].split(",")[-1].strip() == "true", before
+
+
+def test_barriers_are_invalidated_before_their_memory_is_used_again():
+    """A batched CTA calls adj_accumulate once per item: its mbarriers' memory is
+    initialised again, and holds the forward's windows in between, which PTX allows
+    only after mbarrier.inval."""
+    _, body = function_body("adj_accumulate")
+    m = re.search(r"if \(!PLAIN && tid == 0\) \{(.*?)\n  \}\s*__syncthreads\(\);\s*return", body, re.S)
+    assert m
+    assert {"mbar_inval(&s_full[i]);", "mbar_inval(&s_empty[i]);"} <= set(
+        re.findall(r"mbar_inval\([^)]*\);", m.group(1)))
+    assert "mbar_wait" not in m.group(1) and "mbar_wait" not in body[m.end():]
