@@ -24,6 +24,7 @@
 // registers, and the CTA reduces them through shared memory in a fixed order;
 // a combine kernel then sums the tiles' spectra R_n S_n in tile order.  No
 // atomics: results are bitwise reproducible.
+#include <cfloat>
 #include <cmath>
 
 #include "pa_internal.cuh"
@@ -175,12 +176,14 @@ __device__ __forceinline__ void sincos2(float2 f, float2 d, float2& c, float2& s
 
 // 2^e, e in [-126, 127]
 __device__ __forceinline__ float pow2i(int e) { return __int_as_float((e + 127) << 23); }
-// the exponent e of a power-of-two scale 2^e that takes values up to mx below
-// 2^(top + 1); 0 for mx = 0, infinite or NaN
+// The exponent e of a power-of-two scale 2^e that takes values up to mx below
+// 2^(top + 1), over the whole range of FP32 (subnormal values, and an mx that
+// overflowed, count as the nearest end of it: they still land within FP16's range);
+// |e| <= 126, so that 2^e and 2^-e are normal.  0 for mx = 0 or NaN.
 __device__ __forceinline__ int scale_exp(float mx, int top) {
-  if (!(mx > 0.0f) || !(mx <= 3.0e38f)) return 0;
-  const int e = ((__float_as_int(mx) >> 23) & 255) - 127;
-  return max(-100, min(100, top - e));
+  if (!(mx > 0.0f)) return 0;
+  const int e = min((__float_as_int(mx) >> 23) & 255, 254) - 127;
+  return max(-126, min(126, top - e));
 }
 
 // Per (tile, sensor): the geometry that needs FP64 (the FP64 pipe takes 64
@@ -236,7 +239,7 @@ __global__ void __launch_bounds__(kFreqThreads) k_freq_prep(const FreqParams P, 
     for (int n = threadIdx.x & 31; n < P.Q; n += 32) {
       const float2 v = P.p[(int64_t)s * P.Q + n];
       const float m = 6.2831855f * fmaf((float)n, fdf, f0) * fmaxf(fabsf(v.x), fabsf(v.y));
-      bad |= !(fabsf(v.x) <= 3.0e38f) || !(fabsf(v.y) <= 3.0e38f);
+      bad |= !(fabsf(v.x) <= FLT_MAX) || !(fabsf(v.y) <= FLT_MAX);
       mx = fmaxf(mx, m);
     }
     mx = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(mx)));
@@ -546,10 +549,10 @@ __global__ void __launch_bounds__(kFreqThreads, 3) k_freq_adjoint_mma(const Freq
       const FreqRef& r = P.refs[(int64_t)tile * P.S + s];
       const float2 R = centre_phase(r.ph0, r.phd, n);  // conj(R_n) = R.x + i R.y
       const float2 pv = P.p[(int64_t)s * P.Q + n];
-      const float ck = P.cks[n] * pow2i(P.scales[s]);
+      const float ck = P.cks[n], scale = pow2i(P.scales[s]);
       const float2 b = cmul(R, pv);
-      br = ck * b.x;
-      bi = ck * b.y;
+      br = (ck * b.x) * scale;  // ck scale alone may be too large
+      bi = (ck * b.y) * scale;
     }
     const int a = tid >> 4, b = tid & 15;
     const int ks = b >> 3, bk = (b >> 2) & 1, j = a >> 2;
@@ -572,13 +575,11 @@ __global__ void __launch_bounds__(kFreqThreads, 3) k_freq_adjoint_mma(const Freq
     const int s = s0 + it / nblk, n0 = (it % nblk) * 256;
     if (n0 == 0) {
       const FreqRef r = P.refs[(int64_t)tile * P.S + s];
-      const float isc = pow2i(-P.scales[s]);
       __syncwarp();
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
         float2 rinv, dt;
         pixel_part2<DIM>(ox[m], oy[m], oz[m], r, inv_c, rinv, dt);
-        rinv = mul2(rinv, dup(isc));
         float2 vr, vi, ur, ui;
         sincos2(dup(4.0f * fdf), dt, vr, vi);
         sincos2(dup(64.0f * fdf), dt, ur, ui);
@@ -595,6 +596,7 @@ __global__ void __launch_bounds__(kFreqThreads, 3) k_freq_adjoint_mma(const Freq
       __syncwarp();
     }
     const uint4* sBf = reinterpret_cast<const uint4*>(sB + (it & 1) * kFreqFragWords) + lane;
+    const float2 isc = dup(pow2i(-P.scales[s]));
     const float2 fv = dup((float)t * fdf), fu = dup(fmaf((float)(n0 + 16 * t), fdf, f0));
 #pragma unroll 1
     for (int gr = 0; gr < 8; ++gr) {
@@ -641,7 +643,7 @@ __global__ void __launch_bounds__(kFreqThreads, 3) k_freq_adjoint_mma(const Freq
         v.y = fmaf(U.re.y, C[j][3], fmaf(U.im.y, C[j][2], v.y));
         if (j < NJ - 1) U = cmul2(U, U4, nu);
       }
-      sA[gr * 256 + tid] = fma2(v, ld(1), sA[gr * 256 + tid]);
+      sA[gr * 256 + tid] = fma2(mul2(v, ld(1)), isc, sA[gr * 256 + tid]);
     }
   }
   constexpr int TX = Tile<DIM>::X, TY = Tile<DIM>::Y, TZ = Tile<DIM>::Z;
@@ -696,7 +698,7 @@ __global__ void __launch_bounds__(kFreqThreads, 2) k_freq_forward_mma(const Freq
       v = P.x[((int64_t)(tg.tz * TZ + lz) * P.ny + (tg.ty * TY + ly)) * P.nx + (tg.tx * TX + lx)];
     sX[p] = v;
     mx = fmaxf(mx, fabsf(v));
-    bad |= !(fabsf(v) <= 3.0e38f);
+    bad |= !(fabsf(v) <= FLT_MAX);
   }
   mx = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(mx)));
   if (lane == 0) s_max[warp] = mx;
@@ -730,7 +732,7 @@ __global__ void __launch_bounds__(kFreqThreads, 2) k_freq_forward_mma(const Freq
           sincos2(make_float2(-128.0f * fdf, -8.0f * fdf), dt, c, sn);
           __syncwarp();
           wp[lane] = dt.x;
-          wp[32 + lane] = sX[p] * (rinv.x * scale);
+          wp[32 + lane] = (sX[p] * scale) * rinv.x;  // scale alone may be too large
           wp[64 + lane] = c.x;
           wp[96 + lane] = sn.x;
           wp[128 + lane] = c.y;

@@ -1,0 +1,61 @@
+"""The frequency-domain operators from one end of FP32's range to the other: the
+tensor-core kernels scale their FP16 operands by powers of two, which must reach
+every image and spectrum whose result is finite."""
+import numpy as np
+import pytest
+
+from oracle import oracle as orc
+from paper_2404_10928_gb300 import phantoms as ph
+
+from helpers import f32, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+# the FP32 phase error bound of tests/test_gpu_freq.py (1.1e-5 rad at the same
+# f |pixel - tile centre| / c as here), times ten; the scales are powers of two,
+# and what becomes subnormal is below 2^-24 of the largest values
+FREQ_TOL = 1e-4
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2404_10928_gb300 import build
+    build.build()
+    return torch
+
+
+def _problem(unit):
+    """70 x 33 pixels; unit = 1: 0.1 mm and 40 MHz, larger units stretch lengths and
+    times alike (the same phases at frequencies divided by unit)."""
+    sens = np.concatenate([ph.ring_sensors(8, 6e-3), [[0.213e-3, -0.547e-3]]]) * unit
+    return ph.custom(2, (70, 33), (1e-4 * unit, 1e-4 * unit), sens, 64, seed=61, fs=40e6 / unit)
+
+
+# unit, exponents of the image's and of the spectrum's scale.  Stretched by 2^21,
+# frequencies reach 9.5 Hz and distances 20 km, so terms near the top of the range
+# (an image of 2^125 over d, spectra of 2^119 times c k_n) still have finite sums.
+CASES = [(1, -122, -122), (1, 60, 60), (2 ** 21, 0, 0), (2 ** 21, -105, -118), (2 ** 21, 125, 119)]
+
+
+@pytest.mark.parametrize("unit,ex,ep", CASES)
+def test_freq_over_the_range_of_fp32(torch_cuda, unit, ex, ep):
+    torch = torch_cuda
+    from paper_2404_10928_gb300.api import Plan
+    prob = _problem(unit)
+    geo = orc.Geometry.of(prob)
+    q, df = 96, 20e6 / 96 / unit
+    rng = np.random.default_rng(q)
+    x = f32(prob.x_true)
+    pq = rng.standard_normal((prob.n_sensors, q)) + 1j * rng.standard_normal((prob.n_sensors, q))
+    pq = pq.astype(np.complex64).astype(np.complex128)
+    with Plan.from_problem(prob) as plan:
+        xt = torch.tensor(x * 2.0 ** ex, dtype=torch.float32, device="cuda")
+        pt = torch.tensor(pq * 2.0 ** ep, dtype=torch.complex64, device="cuda")
+        p = plan.freq_forward(xt, q, df, df).cpu().numpy().astype(np.complex128)
+        g = plan.freq_adjoint(pt, q, df, df).cpu().numpy().astype(np.float64)
+        plan.sync_status()
+    assert rel_l2(p * 2.0 ** -ex, orc.freq_forward(geo, x, q, df, df)) <= FREQ_TOL
+    assert rel_l2(g * 2.0 ** -ep, orc.freq_adjoint(geo, pq, q, df, df)) <= FREQ_TOL
