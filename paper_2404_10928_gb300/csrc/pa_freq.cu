@@ -14,8 +14,9 @@
 // complex recurrence E_{n+1} = E_n W, W = exp(-i df 2 pi (d - d_ref) / c),
 // re-anchored with sincospi every kAnchor steps.
 //
-// From kMmaForward / kMmaAdjoint frequencies on, the sums run on the tensor cores
-// (see "tensor-core kernels" below); with fewer, by the recurrence:
+// From kMmaForward / kMmaAdjoint frequencies on, reaching phases of kMmaMinSpan
+// cycles across a tile, the sums run on the tensor cores (see "tensor-core kernels"
+// below); else by the recurrence:
 // the adjoint is a gather: each thread accumulates, over the CTA's sensors and
 // all frequencies, Im(conj(E_n) B_n) with B_n = c k_n conj(R_n) P[m][n] staged
 // in shared memory.  Sensor chunks write partial images summed afterwards in
@@ -24,6 +25,7 @@
 // registers, and the CTA reduces them through shared memory in a fixed order;
 // a combine kernel then sums the tiles' spectra R_n S_n in tile order.  No
 // atomics: results are bitwise reproducible.
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 
@@ -253,9 +255,8 @@ __device__ __forceinline__ float2 centre_phase(unsigned long long ph0, unsigned 
                                                int n) {
   const unsigned long long ph = ph0 + (unsigned long long)n * phd;
   const float r = (float)(int)(unsigned)(ph >> 32) * 2.3283064365386963e-10f;
-  float2 c, s;
-  sincos2(dup(r), dup(1.0f), c, s);
-  return make_float2(c.x, s.x);
+  const float2 e = expm2pi(r);
+  return make_float2(e.x, -e.y);
 }
 
 // ------------------------------- adjoint ---------------------------------
@@ -414,20 +415,25 @@ __global__ void __launch_bounds__(kFreqThreads) k_freq_forward(const FreqParams 
 //   adjoint  v_i  = sum_a Im(U_ia sum_b V_ib B_ab)     (contraction over b).
 // Operands go to mma.sync as FP16 pairs hi + lo (22 significant bits of a
 // factor of modulus at most 1; x / d and B scaled by a power of two per (tile,
-// sensor) and per sensor), three products hi hi + hi lo + lo hi with FP32
-// accumulators.  The factors come from one sine and cosine of a phase reduced
-// with one rounding and at most three complex products (the recurrence
-// multiplies up to 32), so the error against FP64 stays that of the FP32 dt:
-// 4.6e-6 to 6e-6 at 256 frequencies on 64^2 to 256^2 grids, forward and adjoint,
-// against 5.3e-6 to 6.4e-6 with the recurrence, and not above it at any count
-// from 4 to 1000.
+// sensor) and per sensor), three products hi hi + hi lo + lo hi.  An MMA adds to its
+// accumulator without rounding to nearest, so the forward's partial sums leave the
+// tensor core after every 16 pixels and are added in FP32.  The factors come from
+// one sine and cosine of a phase reduced with one rounding and at most three complex
+// products (the recurrence multiplies up to 32), so the error against FP64 stays
+// that of the FP32 dt: 5.1e-6 at 256 frequencies up to 20 MHz (96 x 75 pixels of
+// 0.1 mm) in the forward and 4.9e-6 in the adjoint, against 6.4e-6 and 6.1e-6 with
+// the recurrence; at 128 frequencies up to 2 MHz 5.5e-7 and 5.3e-7 against 5.8e-7
+// and 6.5e-7; 5.7e-6 against 6.0e-6 for a positive image up to 20 MHz, and 2e-7 in
+// its lowest rows with both.  (With sums kept in the tensor core over 128
+// pixels, and hi cut in both operands, sums of like terms were off by 2e-6 at any
+// frequency.)
 //
 // What bounds them: issue slots.  Per 16 pixels and sensor a warp issues about
 // 200 instructions for the factors, their splits and the dot products, and 24
 // MMAs, each of which holds the issue port for about 8 cycles (a loop of one
 // m16n8k16 with 4 or 8 independent FFMAs takes 11.6 and 15.9 cycles per step, 8.1
 // without them); the two add up to 92-96% of the measured cycles.  256^2 ring,
-// 256 sensors, 256 frequencies: forward 1470 -> 524 us, adjoint 1266 -> 418 us.
+// 256 sensors, 256 frequencies: forward 1474 -> 553 us, adjoint 1269 -> 429 us.
 struct C2 {  // two complex numbers
   float2 re, im;
 };
@@ -452,6 +458,15 @@ __device__ __forceinline__ void split(float2 v, uint32_t& hi, uint32_t& lo) {
   const float2 h = make_float2(cut(v.x), cut(v.y));
   const float2 r = fma2(h, dup(-1.0f), v);
   hi = pack_h2(h.x, h.y);
+  lo = pack_h2(r.x, r.y);
+}
+// The same with hi rounded to nearest, so that lo carries no sign of its own: one
+// operand of each product is split this way, or the dropped lo lo products, all of
+// one sign, would add up in a sum of like terms.
+__device__ __forceinline__ void split_rn(float2 v, uint32_t& hi, uint32_t& lo) {
+  const __half2 h = __floats2half2_rn(v.x, v.y);
+  const float2 r = fma2(__half22float2(h), dup(-1.0f), v);
+  hi = h2_bits(h);
   lo = pack_h2(r.x, r.y);
 }
 // two complex numbers: (re, im) of number x and of number y
@@ -557,8 +572,8 @@ __global__ void __launch_bounds__(kFreqThreads, 3) k_freq_adjoint_mma(const Freq
     const int a = tid >> 4, b = tid & 15;
     const int ks = b >> 3, bk = (b >> 2) & 1, j = a >> 2;
     uint32_t hi0, lo0, hi1, lo1;
-    split(make_float2(br, -bi), hi0, lo0);
-    split(make_float2(bi, br), hi1, lo1);
+    split_rn(make_float2(br, -bi), hi0, lo0);
+    split_rn(make_float2(bi, br), hi1, lo1);
     uint32_t* buf = sB + (it & 1) * kFreqFragWords;
     const int idx = ks * 8 + j * 2 + bk, ln = 8 * (a & 3) + (b & 3);  // lanes of columns 2a', 2a'+1
     const int w0 = ((idx >> 2) * 32 + ln) * 4 + (idx & 3);
@@ -668,16 +683,16 @@ __global__ void __launch_bounds__(kFreqThreads, 3) k_freq_adjoint_mma(const Freq
 }
 constexpr int kFreqAdjSmem = 2 * kFreqFragWords * 4 + 8 * 6 * 128 * 4 + 8 * 256 * 8;
 
-// Forward.  CTA: one (tile, sensor) pair, 128 pixels per warp (an MMA adds its
-// products to the accumulator without rounding to nearest, so the eight partial
-// sums of 128 pixels, added in FP32, also keep the error at that of an FP32 sum:
-// with one warp per pair it was up to 1.4x larger).  Rows of the A operand are
-// (Re, Im) of x / d U_ia (16-row tile mt: Re of a = 8 mt + g in row g, Im in row
-// g + 8), columns of B are (Re, Im) of V_ib, k runs over 16 pixels: lane 4 g + t
-// generates a, b = g and g + 8 for pixels 2t, 2t + 1, 2t + 8, 2t + 9.  MT = 1 covers
-// up to 128 frequencies per block (a < 8), MT = 2 up to 256.
+// Forward.  CTA: one (tile, sensor) pair, 128 pixels per warp, the warps' sums added
+// in order.  Rows of the A operand are (Re, Im) of x / d U_ia (16-row tile mt: Re of
+// a = 8 mt + g in row g, Im in row g + 8), columns of B are (Re, Im) of V_ib, k runs
+// over 16 pixels: lane 4 g + t generates a, b = g and g + 8 for pixels 2t, 2t + 1,
+// 2t + 8, 2t + 9.  MT = 1 covers up to 128 frequencies per block (a < 8), three CTAs
+// per SM (434 -> 419 us at 128 frequencies); MT = 2 up to 256, two (three spill: 564
+// against 550 us).
 template <int DIM, int MT>
-__global__ void __launch_bounds__(kFreqThreads, 2) k_freq_forward_mma(const FreqParams P) {
+__global__ void __launch_bounds__(kFreqThreads, MT == 1 ? 3 : 2)
+    k_freq_forward_mma(const FreqParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   float* sX = reinterpret_cast<float*>(smem);          // [1024]
   float* sP = sX + kTilePixels;                        // [8 warps][6][32]
@@ -713,11 +728,11 @@ __global__ void __launch_bounds__(kFreqThreads, 2) k_freq_forward_mma(const Freq
   float* wp = sP + warp * 6 * 32;
   constexpr int kBlk = 128 * MT;
   for (int n0 = 0; n0 < P.Q; n0 += kBlk) {
-    float acc[MT][4][4];
+    float2 acc[MT][4][2];
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.0f;
+      for (int j = 0; j < 4; ++j) acc[m][j][0] = acc[m][j][1] = dup(0.0f);
     const float2 fu = dup(-fmaf((float)(n0 + 16 * g), fdf, f0)), fv = dup(-(float)g * fdf);
     if (mx > 0.0f || bad) {
 #pragma unroll 1
@@ -753,13 +768,13 @@ __global__ void __launch_bounds__(kFreqThreads, 2) k_freq_forward_mma(const Freq
             sincos2(fu, dt, U.re, U.im);
             U.re = mul2(U.re, xc);
             U.im = mul2(U.im, xc);
-            split(U.re, Ah[0][2 * h], Al[0][2 * h]);
-            split(U.im, Ah[0][2 * h + 1], Al[0][2 * h + 1]);
+            split_rn(U.re, Ah[0][2 * h], Al[0][2 * h]);
+            split_rn(U.im, Ah[0][2 * h + 1], Al[0][2 * h + 1]);
             if (MT == 2) {
               const C2 U8{ld(2, h), ld(3, h)};
               U = cmul2(U, U8, neg2(U8.im));
-              split(U.re, Ah[MT - 1][2 * h], Al[MT - 1][2 * h]);
-              split(U.im, Ah[MT - 1][2 * h + 1], Al[MT - 1][2 * h + 1]);
+              split_rn(U.re, Ah[MT - 1][2 * h], Al[MT - 1][2 * h]);
+              split_rn(U.im, Ah[MT - 1][2 * h + 1], Al[MT - 1][2 * h + 1]);
             }
             sincos2(fv, dt, V[h].re, V[h].im);
             const C2 V8{ld(4, h), ld(5, h)};
@@ -769,12 +784,18 @@ __global__ void __launch_bounds__(kFreqThreads, 2) k_freq_forward_mma(const Freq
             uint32_t h0, l0, h1, l1;
             split(v0, h0, l0);
             split(v1, h1, l1);
+            float d[MT][4] = {};  // the products of these 16 pixels alone
 #pragma unroll
-            for (int m = 0; m < MT; ++m) mma_f16(acc[m][j], Al[m], h0, h1);
+            for (int m = 0; m < MT; ++m) mma_f16(d[m], Al[m], h0, h1);
 #pragma unroll
-            for (int m = 0; m < MT; ++m) mma_f16(acc[m][j], Ah[m], l0, l1);
+            for (int m = 0; m < MT; ++m) mma_f16(d[m], Ah[m], l0, l1);
 #pragma unroll
-            for (int m = 0; m < MT; ++m) mma_f16(acc[m][j], Ah[m], h0, h1);
+            for (int m = 0; m < MT; ++m) mma_f16(d[m], Ah[m], h0, h1);
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+              acc[m][j][0] = add2(acc[m][j][0], make_float2(d[m][0], d[m][1]));
+              acc[m][j][1] = add2(acc[m][j][1], make_float2(d[m][2], d[m][3]));
+            }
           };
           col(0, V[0].re, V[1].re);
           col(1, V[0].im, V[1].im);
@@ -791,7 +812,8 @@ __global__ void __launch_bounds__(kFreqThreads, 2) k_freq_forward_mma(const Freq
       for (int j = 0; j < 4; ++j)
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-          sR[(warp * 16 * MT + (m * 4 + j) * 4 + e) * 32 + lane] = acc[m][j][e];
+          sR[(warp * 16 * MT + (m * 4 + j) * 4 + e) * 32 + lane] =
+              e & 1 ? acc[m][j][e >> 1].y : acc[m][j][e >> 1].x;
     __syncthreads();
     if (warp < 4 * MT) {
       const int m = warp >> 2, bh = (warp >> 1) & 1, e = warp & 1;
@@ -824,6 +846,25 @@ int freq_fwd_smem(int mt) {
 // at 32, 294 / 262 at 48.  (On small grids the matrix kernels win at any count,
 // by at most 30%: 64^2, 64 sensors, 32 frequencies: 25 against 37 us.)
 constexpr int kMmaForward = 72, kMmaAdjoint = 44;
+// They also take over only where the phases of a tile's pixels span a few cycles at
+// the highest frequency.  Below, the FP32 dt no longer dominates the error, and with
+// few roundings per term the recurrence is up to 1.2x more accurate (96 x 75 pixels
+// of 0.1 mm, 128 and 256 frequencies up to 0.1 MHz, 0.15 cycles: forward 8.3e-8 to
+// 9.4e-8 against 8.9e-8 to 1.1e-7; 1 MHz, 1.5 cycles: 0.9x to 1.2x; 2 MHz, 2.9
+// cycles: 0.97x; adjoint 0.5x to 1.2x, 0.6x to 1.1x and 0.8x).
+constexpr double kMmaMinSpan = 2.5;
+
+// cycles from the centre of a tile to its corner at the highest frequency
+double freq_span(const pa_plan* p, int Q, double f0, double df) {
+  const bool d2 = p->dim == 2;
+  const double ex = (std::min(p->grid.nx, d2 ? Tile<2>::X : Tile<3>::X) - 1) * p->grid.dx;
+  const double ey = (std::min(p->grid.ny, d2 ? Tile<2>::Y : Tile<3>::Y) - 1) * p->grid.dy;
+  const double ez = d2 ? 0.0 : (std::min(p->grid.nz, Tile<3>::Z) - 1) * p->grid.dz;
+  return 0.5 * std::sqrt(ex * ex + ey * ey + ez * ez) / p->c * (f0 + (Q - 1) * df);
+}
+bool use_mma(const pa_plan* p, int Q, double f0, double df, int min_count) {
+  return Q >= min_count && freq_span(p, Q, f0, df) >= kMmaMinSpan;
+}
 
 __global__ void __launch_bounds__(kFreqThreads) k_freq_combine(const FreqParams P, int ntiles) {
   const int64_t idx = blockIdx.x * (int64_t)kFreqThreads + threadIdx.x;
@@ -950,7 +991,7 @@ pa_status pa_freq_forward(pa_plan* plan, int n_freq, double f0, double df, const
                           float* p_dev, pa_stream stream) {
   PA_TRY(check_freq(plan, n_freq, f0, df, x_dev, p_dev, "pa_freq_forward"));
   DeviceGuard guard(plan->device);
-  const bool mma = n_freq >= kMmaForward;
+  const bool mma = use_mma(plan, n_freq, f0, df, kMmaForward);
   const size_t bytes = (size_t)plan->S * plan->ntiles * n_freq * sizeof(float2);
   PA_TRY(freq_workspace(plan, a256(bytes) + freq_table_bytes(plan, n_freq)));
   FreqParams f = freq_params(plan, n_freq, f0, df);
@@ -996,7 +1037,7 @@ pa_status pa_freq_adjoint(pa_plan* plan, int n_freq, double f0, double df, const
     set_error("pa_freq_adjoint: n_freq %d needs more shared memory than a CTA has", n_freq);
     return PA_ERR_UNSUPPORTED;
   }
-  const bool mma = n_freq >= kMmaAdjoint;
+  const bool mma = use_mma(plan, n_freq, f0, df, kMmaAdjoint);
   if (mma) {
     // fewer sensors per CTA until the grid fills the chip
     f.spc = kFreqSensors;

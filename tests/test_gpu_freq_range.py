@@ -59,3 +59,39 @@ def test_freq_over_the_range_of_fp32(torch_cuda, unit, ex, ep):
         plan.sync_status()
     assert rel_l2(p * 2.0 ** -ex, orc.freq_forward(geo, x, q, df, df)) <= FREQ_TOL
     assert rel_l2(g * 2.0 ** -ep, orc.freq_adjoint(geo, pq, q, df, df)) <= FREQ_TOL
+
+
+def _coherent_problem():
+    # a positive image: the terms of a sum at low frequencies all have one sign
+    prob = ph.custom(2, (96, 75), (1e-4, 1e-4), ph.ring_sensors(8, 8e-3), 64, seed=63)
+    prob.x_true = 1.0 + 0.1 * prob.x_true
+    return prob
+
+
+def _coherent_tol(f):
+    """FP32 phases 2 pi s 2^-24 (s = cycles from a tile's centre to its corner, 1.46
+    us of travel), plus in units of 2^-24: two sines within 1.5e-7 (5), operands as
+    pairs of 22 bits (4), and the FP32 sums (3)."""
+    return (2.0 * np.pi * 1.46e-6 * f + 12.0) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("q", [100, 200])
+@pytest.mark.parametrize("fmax", [0.1e6, 0.7e6, 1.6e6, 1.8e6, 20e6])
+def test_forward_of_like_terms_has_the_error_of_fp32(torch_cuda, q, fmax):
+    torch = torch_cuda
+    from paper_2404_10928_gb300.api import Plan
+    prob = _coherent_problem()
+    geo = orc.Geometry.of(prob)
+    df = fmax / q
+    x = f32(prob.x_true)
+    with Plan.from_problem(prob) as plan:
+        p = plan.freq_forward(torch.tensor(x, dtype=torch.float32, device="cuda"), q, df, df)
+        p = p.cpu().numpy()
+        plan.sync_status()
+    ref = orc.freq_forward(geo, x, q, df, df)
+    # the spectra up to 0.5 MHz (0.7 cycles, where a tile's sum does not cancel)
+    low = [n for n in range(q) if (n + 1) * df <= 0.5e6]
+    assert low
+    for n in low[:3] + low[-3:]:
+        err = rel_l2(p[:, n], ref[:, n])
+        assert err <= _coherent_tol((n + 1) * df), (n, err)
