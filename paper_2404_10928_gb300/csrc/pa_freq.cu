@@ -853,6 +853,10 @@ constexpr int kMmaForward = 72, kMmaAdjoint = 44;
 // 9.4e-8 against 8.9e-8 to 1.1e-7; 1 MHz, 1.5 cycles: 0.9x to 1.2x; 2 MHz, 2.9
 // cycles: 0.97x; adjoint 0.5x to 1.2x, 0.6x to 1.1x and 0.8x).
 constexpr double kMmaMinSpan = 2.5;
+// And not where sincos2's phases could leave its domain of 2^21 cycles (the blocks
+// reach up to twice the highest frequency): such phases mean little in FP32, but the
+// recurrence's factors keep their modulus of 1.
+constexpr double kMmaMaxSpan = 524288.0;
 
 // cycles from the centre of a tile to its corner at the highest frequency
 double freq_span(const pa_plan* p, int Q, double f0, double df) {
@@ -863,7 +867,8 @@ double freq_span(const pa_plan* p, int Q, double f0, double df) {
   return 0.5 * std::sqrt(ex * ex + ey * ey + ez * ez) / p->c * (f0 + (Q - 1) * df);
 }
 bool use_mma(const pa_plan* p, int Q, double f0, double df, int min_count) {
-  return Q >= min_count && freq_span(p, Q, f0, df) >= kMmaMinSpan;
+  const double span = freq_span(p, Q, f0, df);
+  return Q >= min_count && span >= kMmaMinSpan && span <= kMmaMaxSpan;
 }
 
 __global__ void __launch_bounds__(kFreqThreads) k_freq_combine(const FreqParams P, int ntiles) {

@@ -95,3 +95,29 @@ def test_forward_of_like_terms_has_the_error_of_fp32(torch_cuda, q, fmax):
     for n in low[:3] + low[-3:]:
         err = rel_l2(p[:, n], ref[:, n])
         assert err <= _coherent_tol((n + 1) * df), (n, err)
+
+
+@pytest.mark.parametrize("span", [2.0 ** 16, 2.0 ** 20, 2.0 ** 24, 2.0 ** 28])
+def test_phases_of_many_cycles_keep_the_modulus(torch_cuda, span):
+    """With more cycles across a tile than FP32 resolves, the phases carry no
+    information, but every term keeps its modulus: |P| <= c k sum |x| / d."""
+    torch = torch_cuda
+    from paper_2404_10928_gb300.api import Plan
+    prob = _problem(1)
+    q = 200
+    df = span / 1.5e-6 / q
+    rng = np.random.default_rng(q)
+    x = f32(prob.x_true)
+    pq = (rng.standard_normal((9, q)) + 1j * rng.standard_normal((9, q))).astype(np.complex64)
+    with Plan.from_problem(prob) as plan:
+        p = plan.freq_forward(torch.tensor(x, dtype=torch.float32, device="cuda"), q, df, df)
+        g = plan.freq_adjoint(torch.tensor(pq, device="cuda"), q, df, df)
+        p, g = p.cpu().numpy(), g.cpu().numpy()
+        plan.sync_status()
+    o = np.asarray(prob.origin[:2])
+    pix = np.stack(np.meshgrid(np.arange(70) * 1e-4 + o[0], np.arange(33) * 1e-4 + o[1]), -1)
+    inv_d = 1.0 / np.linalg.norm(pix.reshape(-1, 1, 2) - prob.sensors[None], axis=2)  # [N][S]
+    ck = 2.0 * np.pi * df * (1 + np.arange(q))
+    # FP32 factors: moduli within 32 recurrence steps of 2^-22, rounded up
+    assert (np.abs(p) <= 1.001 * (x @ inv_d)[:, None] * ck).all()
+    assert (np.abs(g) <= 1.001 * (inv_d @ (np.abs(pq) @ ck))).all()
