@@ -557,7 +557,9 @@ cudaError_t launch_build_table(int dim, TileRef* table, int2* krange, const doub
 // pa_plan_set_sound_speed: 0.40 -> 0.08 ms at 256^2 with 128 sensors, 95 -> 9.6 ms at
 // 128^3 with 1024 (creating that plan: 97 -> 11 ms).
 constexpr int kOrderThreads = 256;
-constexpr int kOrderStaged = 12 * 1024;  // entries (48 KB)
+// entries staged: 48 KB, the default limit of a launch's shared memory, less room for
+// the kernel's own (s_warp)
+constexpr int kOrderStaged = 12 * 1024 - 64;
 __global__ void __launch_bounds__(kOrderThreads) k_combine_order(const TileRef* table, int2* sorted,
                                                                  int* upper, int S, int K, int L,
                                                                  int ntiles, int staged) {
