@@ -35,7 +35,8 @@ from torch.utils.checkpoint import checkpoint
 
 
 def _value(c) -> float:
-    return float(c.detach())
+    """The speed of sound as a number: from a tensor, or a number that takes no gradient."""
+    return float(c.detach() if isinstance(c, torch.Tensor) else c)
 
 
 def _set_c(plan, cv: float) -> None:
