@@ -223,9 +223,10 @@ class UnrolledLandweber(torch.nn.Module):
 
     def forward(self, x0, y, c):
         x = x0
-        # an overridden step takes (x, y, c) and may draw random numbers; the
-        # class's own takes the value of c, read once, and draws none
-        own = type(self).step is UnrolledLandweber.step
+        # a replaced step (of a subclass or of this instance) takes (x, y, c) and may
+        # draw random numbers; the class's own takes the value of c, read once, and
+        # draws none
+        own = getattr(self.step, "__func__", None) is UnrolledLandweber.step
         args = (y, c, _value(c)) if own else (y, c)
         for _ in range(self.n_iter):
             if self.checkpointing:

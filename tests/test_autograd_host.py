@@ -52,3 +52,51 @@ def test_speed_of_sound_as_a_number(c):
     for checkpointing in (False, True):
         net = autograd.UnrolledLandweber(plan, 1, 0.1, checkpointing=checkpointing)
         assert torch.equal(net(x, y, c), step)
+
+
+@pytest.mark.parametrize("checkpointing", [False, True])
+@pytest.mark.parametrize("how", ["instance", "subclass"])
+def test_replaced_step_takes_x_y_c_and_keeps_its_random_numbers(checkpointing, how):
+    plan = DensePlan()
+    c = torch.tensor(1500.0)
+    y = torch.rand((1, plan.n_sensors, plan.n_samples))
+    keep = []
+
+    def step(x, y, c):
+        # a step with random numbers: recomputing it in backward must draw the same
+        mask = (torch.rand_like(x) < 0.5).to(x.dtype)
+        keep.append(mask)
+        return x * x * mask
+
+    if how == "instance":
+        net = autograd.UnrolledLandweber(plan, 2, 0.1, checkpointing=checkpointing)
+        net.step = step
+    else:
+        class Net(autograd.UnrolledLandweber):
+            def step(self, x, y, c):
+                return step(x, y, c)
+        net = Net(plan, 2, 0.1, checkpointing=checkpointing)
+    x = torch.rand((1, plan.n_pixels), requires_grad=True)
+    torch.manual_seed(5)
+    out = net(x, y, c)
+    m1, m2 = keep[:2]
+    torch.manual_seed(6)  # backward runs with another state of the generator
+    out.sum().backward()
+    # out = m2 (m1 x^2)^2
+    assert torch.allclose(x.grad, 4.0 * m2 * m1 * x.detach() ** 3)
+
+
+def test_wrapped_bound_step_is_a_replacement():
+    plan = DensePlan()
+    net = autograd.UnrolledLandweber(plan, 3, 0.1)
+    own, calls = net.step, []
+
+    def traced(x, y, c):
+        calls.append(float(c))
+        return own(x, y, c)
+
+    x, y = torch.rand((1, plan.n_pixels)), torch.rand((1, plan.n_sensors, plan.n_samples))
+    expect = net(x, y, torch.tensor(1510.0))
+    net.step = traced
+    assert torch.equal(net(x, y, torch.tensor(1510.0)), expect)
+    assert calls == [1510.0] * 3
