@@ -104,7 +104,10 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_mv(const T* m, const T*
     const V* vv = reinterpret_cast<const V*>(v);
     const int64_t n = cols / VW;
     int64_t j = threadIdx.x;
-    for (; j + 3 * kDenseThreads < n; j += 4 * kDenseThreads) {
+    // rounds that every lane of the warp has, so that all of them vote; a lane's
+    // further entries follow one by one, in the same order
+    const int64_t whole = n - 3 * kDenseThreads - (31 - (threadIdx.x & 31));
+    for (; j < whole; j += 4 * kDenseThreads) {
       V a[4], b[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -115,7 +118,7 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_mv(const T* m, const T*
         bool any = false;
 #pragma unroll
         for (int u = 0; u < 4; ++u) any |= counts(a[u].x, b[u].x) | counts(a[u].y, b[u].y);
-        if (!__any_sync(__activemask(), any)) continue;
+        if (!__any_sync(0xffffffffu, any)) continue;
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) dot(a[u], b[u]);
@@ -146,27 +149,30 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_mtv(const T* m, const T
   const int64_t r1 = min(rows, r0 + kRowsPerChunk);
   if (c < cols) {
     T acc = 0;
+    int64_t r = r0;
     if constexpr (sizeof(T) == 8) {
-      // rounds of eight rows, loaded before the tests decide
+      // rounds of eight rows, loaded before the tests decide; a warp that the last
+      // column cuts off skips nothing, so that all lanes vote
       constexpr int U = 8;
-      int64_t r = r0;
-      for (; r + U <= r1; r += U) {
-        T a[U], b[U];
+      if (c - (threadIdx.x & 31) + 32 <= cols) {
+        for (; r + U <= r1; r += U) {
+          T a[U], b[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          a[u] = __ldcs(m + (r + u) * cols + c);
-          b[u] = __ldg(v + r + u);
+          for (int u = 0; u < U; ++u) {
+            a[u] = __ldcs(m + (r + u) * cols + c);
+            b[u] = __ldg(v + r + u);
+          }
+          bool any = false;
+#pragma unroll
+          for (int u = 0; u < U; ++u) any |= counts(a[u], b[u]);
+          if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
+          for (int u = 0; u < U; ++u) acc = fma(a[u], b[u], acc);
         }
-        bool any = false;
-#pragma unroll
-        for (int u = 0; u < U; ++u) any |= counts(a[u], b[u]);
-        if (!__any_sync(__activemask(), any)) continue;
-#pragma unroll
-        for (int u = 0; u < U; ++u) acc = fma(a[u], b[u], acc);
       }
       for (; r < r1; ++r) acc = fma(__ldcs(m + r * cols + c), __ldg(v + r), acc);
     } else {
-      for (int64_t r = r0; r < r1; ++r) acc += __ldcs(m + r * cols + c) * __ldg(v + r);
+      for (; r < r1; ++r) acc += __ldcs(m + r * cols + c) * __ldg(v + r);
     }
     part[(int64_t)blockIdx.y * cols + c] = acc;
   }
