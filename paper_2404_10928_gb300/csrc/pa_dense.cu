@@ -12,14 +12,15 @@
 // thread per pair writing its two entries, evaluated in FP64 with the
 // oracle's operation order (no FMA contraction) and rounded once for FP32.
 // The products are bound by HBM (one pass over M).  In FP64 one FMA per entry would
-// bind them to GB300's FP64 pipe (~64 cycles per warp instruction: 189 and 182 us at
-// 6144 x 16384, against 118 us for the bytes at 6.8 TB/s); a measurement matrix is
-// mostly zeros (two entries per pixel and sensor), so a round of entries that are
-// all zero for a warp and meet finite vector values, which would leave the sums as
-// they are, is skipped on integer tests: both products together 374 -> 255 us (237
-// for the bytes).  A matrix without zeros pays the tests (190 to 191 and 183 to 188
-// us).  (Skipped one by one, the FMAs are predicated and still take their turn in
-// the pipe.)  Every sum runs in a fixed order, so results are bitwise reproducible.
+// bind them to GB300's FP64 pipe (~64 cycles per warp instruction: M x 194 and M^T r
+// 187 us at 6144 x 16384, against 118 us for the bytes at 6.8 TB/s); a measurement
+// matrix is mostly zeros (two entries per pixel and sensor), so a round of entries
+// that are all zero for a warp and meet finite vector values, which would leave the
+// sums as they are, is skipped on integer tests: 124 and 135 us.  M^T r tests its
+// CTA's share of the vector once (161 us with that test in every round of eight); a
+// matrix without zeros pays little for the tests (194 and 189 us).  (Skipped one by
+// one, the FMAs are predicated and still take their turn in the pipe.)  Every sum
+// runs in a fixed order, so results are bitwise reproducible.
 #include "pa_internal.cuh"
 
 namespace pa {
@@ -59,10 +60,13 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_taps(
 
 // Whether a product a b can change a sum that started at +0 (and so never is -0):
 // a is not +-0, or b is infinite or NaN.  Integer tests keep off the FP64 pipe.
-__device__ __forceinline__ bool counts(double a, double b) {
-  return ((__double2hiint(a) << 1) | __double2loint(a)) != 0 ||
-         (__double2hiint(b) & 0x7ff00000) == 0x7ff00000;
+__device__ __forceinline__ bool not_zero(double a) {
+  return ((__double2hiint(a) & 0x7fffffff) | __double2loint(a)) != 0;
 }
+__device__ __forceinline__ bool is_finite(double b) {
+  return (__double2hiint(b) & 0x7ff00000) != 0x7ff00000;
+}
+__device__ __forceinline__ bool counts(double a, double b) { return not_zero(a) || !is_finite(b); }
 
 template <typename T>
 __device__ __forceinline__ T block_sum_t(T v, T* s_red) {
@@ -147,13 +151,19 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_mtv(const T* m, const T
   const int64_t c = blockIdx.x * (int64_t)kDenseThreads + threadIdx.x;
   const int64_t r0 = (int64_t)blockIdx.y * kRowsPerChunk;
   const int64_t r1 = min(rows, r0 + kRowsPerChunk);
+  // v's share of this CTA finite: then only zeros of M decide what can be skipped
+  bool finite = true;
+  if constexpr (sizeof(T) == 8) {
+    const int64_t rv = r0 + threadIdx.x;
+    finite = __syncthreads_or(threadIdx.x < kRowsPerChunk && rv < r1 && !is_finite(__ldg(v + rv))) == 0;
+  }
   if (c < cols) {
     T acc = 0;
     int64_t r = r0;
     if constexpr (sizeof(T) == 8) {
-      // rounds of eight rows, loaded before the tests decide; a warp that the last
+      // rounds of 16 rows, loaded before the test decides; a warp that the last
       // column cuts off skips nothing, so that all lanes vote
-      constexpr int U = 8;
+      constexpr int U = 16;
       if (c - (threadIdx.x & 31) + 32 <= cols) {
         for (; r + U <= r1; r += U) {
           T a[U], b[U];
@@ -162,10 +172,11 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_mtv(const T* m, const T
             a[u] = __ldcs(m + (r + u) * cols + c);
             b[u] = __ldg(v + r + u);
           }
-          bool any = false;
+          bool any = !finite;
 #pragma unroll
-          for (int u = 0; u < U; ++u) any |= counts(a[u], b[u]);
+          for (int u = 0; u < U; ++u) any |= not_zero(a[u]);
           if (!__any_sync(0xffffffffu, any)) continue;
+          __syncwarp();  // keeps this a branch: predicated, the FMAs take their turn in the pipe
 #pragma unroll
           for (int u = 0; u < U; ++u) acc = fma(a[u], b[u], acc);
         }
