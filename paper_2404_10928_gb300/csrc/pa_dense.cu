@@ -16,11 +16,11 @@
 // 187 us at 6144 x 16384, against 118 us for the bytes at 6.8 TB/s); a measurement
 // matrix is mostly zeros (two entries per pixel and sensor), so a round of entries
 // that are all zero for a warp and meet finite vector values, which would leave the
-// sums as they are, is skipped on integer tests: 124 and 135 us.  M^T r tests its
-// CTA's share of the vector once (161 us with that test in every round of eight); a
-// matrix without zeros pays little for the tests (194 and 189 us).  (Skipped one by
-// one, the FMAs are predicated and still take their turn in the pipe.)  Every sum
-// runs in a fixed order, so results are bitwise reproducible.
+// sums as they are, is skipped on integer tests: 123 and 139 us.  M^T r tests its
+// CTA's share of the vector once (161 us with that test in every round); a matrix
+// without zeros pays for the tests (194 and 195 us).  (Skipped one by one, the FMAs
+// are predicated and still take their turn in the pipe.)  Every sum runs in a fixed
+// order, so results are bitwise reproducible.
 #include "pa_internal.cuh"
 
 namespace pa {
@@ -161,10 +161,14 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_mtv(const T* m, const T
     T acc = 0;
     int64_t r = r0;
     if constexpr (sizeof(T) == 8) {
-      // rounds of 16 rows, loaded before the test decides; a warp that the last
-      // column cuts off skips nothing, so that all lanes vote
-      constexpr int U = 16;
+      // rounds of eight rows, loaded before the test decides; a warp that the last
+      // column cuts off skips nothing, so that all lanes vote.  Unrolled by two (62
+      // registers, 608 CTAs resident) it is within 2% of the best of all sizes tried
+      // (64^2 to 128^2, 24 to 64 sensors, 80 to 160 samples); rounds of 16 take 135
+      // instead of 139 us at 6144 x 16384, but 89 instead of 84 us at 5760 x 10000.
+      constexpr int U = 8;
       if (c - (threadIdx.x & 31) + 32 <= cols) {
+#pragma unroll 2
         for (; r + U <= r1; r += U) {
           T a[U], b[U];
 #pragma unroll
