@@ -45,7 +45,7 @@ WORKLOAD = "2D 256x256 0.1mm, 256-sensor ring R=20mm, 2048 samples @40MHz, c=150
 N_ITER = 50
 FLOPS_PER_PAIR = 18  # 9 FP32 instructions per pair (FFMA-equivalent, 2 flop each)
 MUFU_PER_PAIR = 2    # rsqrt (1/d) and rcp (the difference form of the arrival) per pair
-SFU_PER_SM_CLK = 16  # MUFU results per SM per clock
+SFU_PER_SM_CLK = 16  # rsqrt or rcp results per SM per clock (a loop of either: 15.2)
 L2_FLUSH_BYTES = 256 << 20
 
 

@@ -31,7 +31,8 @@ FWD_SENSORS = (8, 12, 16, 20, 24, 32, 48, 64, 96, 128)
 FWD_THREADS = (64, 128, 256)
 ADJ_WARPS = (4, 8)
 # (adj_cluster, fwd_sensors_per_cta, fwd_threads, adj_warps) held fixed while
-# the other operator's options vary
+# the other operator's options vary (a plan created without options takes its own from
+# its size)
 DEFAULT = (1, 32, 128, 8)
 
 
@@ -51,8 +52,8 @@ def size_key(gpu: str, dim: int, n_pixels: int, n_sensors: int, n_samples: int,
 def candidates(n_sensors: int) -> Iterable[Tuple[int, int, int, int]]:
     """(adj_cluster, fwd_sensors_per_cta, fwd_threads, adj_warps).  The
     cluster and warps only change the adjoint, the other two only the forward,
-    so the forward pair is searched jointly with the adjoint at its defaults,
-    and the adjoint pair with the forward at its defaults."""
+    so the forward pair is searched jointly with the adjoint's held fixed, and
+    the adjoint pair with the forward's held fixed (DEFAULT)."""
     for nt in FWD_THREADS:
         for spc in FWD_SENSORS:
             yield DEFAULT[0], spc, nt, DEFAULT[3]
@@ -114,9 +115,9 @@ class Autotuner:
         timings = {}
         for cand in candidates(prob.n_sensors):
             timings[cand] = float(self.measure(prob, *cand))
-        # the forward pair with the adjoint at its defaults (ties to fewer
-        # threads, then fewer sensors); the adjoint pair with the forward at
-        # its defaults (ties to the smaller cluster, then fewer warps)
+        # the forward pair with the adjoint's held fixed (ties to fewer threads,
+        # then fewer sensors); the adjoint pair with the forward's held fixed (ties
+        # to the smaller cluster, then fewer warps)
         fwd = {(spc, nt): t for (c, spc, nt, aw), t in timings.items()
                if (c, aw) == (DEFAULT[0], DEFAULT[3])}
         spc, nt = min(fwd, key=lambda v: (fwd[v], v[1], v[0]))

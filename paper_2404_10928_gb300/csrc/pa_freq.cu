@@ -197,7 +197,6 @@ __device__ __forceinline__ int scale_exp(float mx, int top) {
 template <int DIM>
 __global__ void __launch_bounds__(kFreqThreads) k_freq_prep(const FreqParams P, int nb_ref,
                                                             int nb_ck) {
-  constexpr int TX = Tile<DIM>::X, TY = Tile<DIM>::Y, TZ = Tile<DIM>::Z;
   const int b = blockIdx.x;
   if (b < nb_ref) {
     const int64_t idx = (int64_t)b * kFreqThreads + threadIdx.x;
@@ -225,9 +224,6 @@ __global__ void __launch_bounds__(kFreqThreads) k_freq_prep(const FreqParams P, 
     r.phd = (unsigned long long)(cd * 18446744073709551616.0);
     r.dlo = (float)fmax(sqrt(qx * qx + qy * qy + qz * qz), 0.45 * hmin);
     P.refs[idx] = r;
-    (void)TX;
-    (void)TY;
-    (void)TZ;
   } else if (b < nb_ref + nb_ck) {
     const int n = (b - nb_ref) * kFreqThreads + threadIdx.x;
     if (n < P.Q) P.cks[n] = (float)(2.0 * M_PI * (P.f0 + n * P.df));  // c k_n
@@ -429,10 +425,10 @@ __global__ void __launch_bounds__(kFreqThreads) k_freq_forward(const FreqParams 
 // frequency.)
 //
 // What bounds them: issue slots.  Per 16 pixels and sensor a warp issues about
-// 200 instructions for the factors, their splits and the dot products, and 24
-// MMAs, each of which holds the issue port for about 8 cycles (a loop of one
-// m16n8k16 with 4 or 8 independent FFMAs takes 11.6 and 15.9 cycles per step, 8.1
-// without them); the two add up to 92-96% of the measured cycles.  256^2 ring,
+// 200 instructions for the factors, their splits and the dot products (220 with the
+// forward's sums), and 24 MMAs, each of which holds the issue port for about 8 cycles
+// (a loop of one m16n8k16 with 4 or 8 independent FFMAs takes 11.6 and 15.9 cycles
+// per step, 8.1 without them); the two add up to 86-89% of the cycles.  256^2 ring,
 // 256 sensors, 256 frequencies: forward 1474 -> 553 us, adjoint 1269 -> 429 us.
 struct C2 {  // two complex numbers
   float2 re, im;
@@ -963,7 +959,8 @@ cudaError_t freq_prep(const pa_plan* p, const FreqParams& f, cudaStream_t st) {
   kernel<<<nb_ref + nb_ck + nb_sc, kFreqThreads, 0, st>>>(f, nb_ref, nb_ck);
   return cudaGetLastError();
 }
-// CTAs that fill the chip (two per SM are resident)
+// CTAs that the adjoint's work split aims at: two per SM.  Three are resident, so a
+// split that just reaches this leaves a third of their places empty.
 int64_t freq_wave() {
   int dev = 0, n = 152;
   if (cudaGetDevice(&dev) != cudaSuccess ||
