@@ -108,10 +108,10 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_mv(const T* m, const T*
     const V* vv = reinterpret_cast<const V*>(v);
     const int64_t n = cols / VW;
     int64_t j = threadIdx.x;
-    // rounds that every lane of the warp has, so that all of them vote; a lane's
-    // further entries follow one by one, in the same order
+    // in FP64, rounds that every lane of the warp has, so that all of them vote; a
+    // lane's further entries follow one by one, in the same order
     const int64_t whole = n - 3 * kDenseThreads - (31 - (threadIdx.x & 31));
-    for (; j < whole; j += 4 * kDenseThreads) {
+    for (; sizeof(T) == 8 ? j < whole : j + 3 * kDenseThreads < n; j += 4 * kDenseThreads) {
       V a[4], b[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
